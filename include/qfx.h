@@ -266,7 +266,7 @@ qfx_status qfx_amplitudes_static(const qfx_plan* p, const uint64_t* x1, int64_t 
  * shapes -- run together:
  * - items whose steps all run FP32 tiles (FP32 plans, and split-precision plans whose
  *   step shapes the tensor-core tile does not take) and whose largest step has fewer
- *   than 512 output tiles: in ONE persistent kernel, a device task queue of fold chunks,
+ *   than 1024 output tiles: in ONE persistent kernel, a device task queue of fold chunks,
  *   scale chunks, contraction-step tiles (each step's plan-chosen variant) and FP64
  *   accumulations, with per-segment completion counters as dependencies and bounded
  *   waits;

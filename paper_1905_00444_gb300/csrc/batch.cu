@@ -101,15 +101,18 @@ __device__ __forceinline__ unsigned long long gtimer() {
 
 __device__ void run_step_tile(const simt::StepArgs& a, int variant, int64_t tile, float4* smem) {
   switch (variant) {
-#define QFX_CASE(V, BM, BJ, TM, TJ, KM, ST) \
-  case V: simt::cgemm_tile<BM, BJ, TM, TJ, KM, ST>(a, tile, 0, smem); break;
+#define QFX_CASE(V, BM, BJ, TM, TJ, KM) \
+  case V: simt::cgemm_tile<BM, BJ, TM, TJ, KM>(a, tile, 0, smem); break;
     QFX_SIMT_VARIANTS(QFX_CASE)
 #undef QFX_CASE
     default: break;
   }
 }
 
-__global__ void __launch_bounds__(kT, 1) batch_kernel(const BatchArgs a) {
+// Two CTAs per SM: while one waits for a dependency or starts a tile the other computes (768
+// items of 4x4x16, 4x5x16 and 5x5x24: 13.5 ms, against 17.4 with one).  The registers that
+// this leaves spill a little around the tile loops.
+__global__ void __launch_bounds__(kT, 2) batch_kernel(const BatchArgs a) {
   extern __shared__ float4 smem[];
   __shared__ long long s_task;
   __shared__ int s_seg, s_go;
@@ -260,7 +263,7 @@ namespace {
 
 size_t batch_smem() {
   size_t m = 0;
-#define QFX_SZ(V, BM, BJ, TM, TJ, KM, ST) m = std::max(m, simt::Cfg<BM, BJ, TM, TJ, KM, ST>::SMEM);
+#define QFX_SZ(V, BM, BJ, TM, TJ, KM) m = std::max(m, simt::Cfg<BM, BJ, TM, TJ, KM>::SMEM);
   QFX_SIMT_VARIANTS(QFX_SZ)
 #undef QFX_SZ
   return m;
@@ -269,7 +272,7 @@ size_t batch_smem() {
 int64_t step_tiles(int variant, int64_t N, int64_t J) {
   int bm = 128, bj = 128;
   switch (variant) {
-#define QFX_T(V, BM, BJ, TM, TJ, KM, ST) case V: bm = BM; bj = BJ; break;
+#define QFX_T(V, BM, BJ, TM, TJ, KM) case V: bm = BM; bj = BJ; break;
     QFX_SIMT_VARIANTS(QFX_T)
 #undef QFX_T
     default: break;
@@ -317,8 +320,9 @@ using namespace qfx;
 // Whether an FP32 work item runs as its own launch sequence in a batch's graph: its
 // largest step has at least kBigTiles output tiles, so the step kernels fill the GPU many
 // times over and launch overhead is negligible, while the same tiles run slower inside the
-// persistent kernel (measured: 48.2 against 41.6 TFLOP/s on the mixed-grid batch).
-constexpr int64_t kBigTiles = 512;
+// persistent kernel (measured with tiles of twice the columns, 512 of which drew the line at
+// the same step sizes: 48.2 against 41.6 TFLOP/s on the mixed-grid batch).
+constexpr int64_t kBigTiles = 1024;
 bool item_is_big(const qfx_plan* p) {
   if (p->family == 1) return true;   // contraction trees run through the launch path only
   int64_t most = 0;

@@ -282,6 +282,27 @@ def test_fill_variants_bit_identical(qfx, shape):
     qfx.sync()
 
 
+@pytest.mark.parametrize("variant", [-1, 5, 6, 7, 8, 9, 25, 26, 27, 28])
+@pytest.mark.parametrize("shape", [(5, 9, 20, 10, 3), (3, 17, 64, 64, 129), (1, 8, 8, 8, 511),
+                                   (131, 7, 66, 22, 5), (129, 33, 70, 35, 1), (2, 1, 2, 1, 7)])
+def test_contract_step_odd_columns(qfx, variant, shape):
+    """Odd Sd: column pairs that straddle two values of p, an odd last column, slabs of one
+    row, and Sd = 1 (columns contiguous in k).  2K fused products per component, each with a
+    relative error of at most 2^-24 of the sum of magnitudes so far: sqrt(2) 2K 2^-24 of
+    sum_k |S||B|, plus the rounding of the result."""
+    P, K, N, NL, Sd = shape
+    S = ri.random_complex((K, N), seed=11)
+    B = ri.random_complex((P, K, Sd), seed=12)
+    order = lambda v: v.reshape(P, N // NL, NL, Sd).transpose(1, 0, 2, 3)  # noqa: E731
+    want = order(primitives.contract_step(S, B, P, K, N, Sd))
+    scale = order(primitives.contract_step(np.abs(S), np.abs(B), P, K, N, Sd).real)
+    out = qfx.contract_step(torch.from_numpy(S.reshape(-1)).cuda(), torch.from_numpy(B.reshape(-1)).cuda(),
+                            P, K, N, NL, Sd, variant=variant)
+    qfx.sync()
+    got = out.cpu().numpy().reshape(want.shape)
+    assert np.all(np.abs(got - want) <= np.sqrt(2.0) * (2 * K + 1) * 2.0 ** -24 * scale)
+
+
 @pytest.mark.parametrize("case", [((4, 5, 6), (2, 0, 1)), ((33, 65), (1, 0)),
                                   ((2, 3, 4, 5, 6), (4, 2, 0, 3, 1)), ((7, 8, 9), (0, 2, 1)),
                                   ((64, 3, 64), (2, 1, 0)), ((5, 1, 7), (1, 2, 0)),
