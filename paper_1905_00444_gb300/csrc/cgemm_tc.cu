@@ -13,26 +13,20 @@
 //   TF32x3: x = b + s, products bb, bs, sb  (error ~2^-21 relative).
 // Accumulation is FP32 in TMEM.
 //
-// Tiles: a persistent CTA per SM walks tiles of 128 columns j (M = 128; the boundary
-// tensor B is the A operand, rows j) by Nt rows n of the site matrix S (the B operand).
-// Default tiles are 128 x 128 with split accumulators in TMEM: hi x hi products go to
-// "main" accumulators (re [0,128), im [128,256)), every cross-term product to "small"
-// ones (re [256,384), im [384,512)), added in the epilogue, so the large accumulators
-// see two additions per k-stage.  There the complex product is embedded in N: S is held
-// per term as planes Sr, Si, -Sr, and one MMA of N = 256 takes Ar x [Sr; Si] into
+// Tiles: the boundary tensor B is the A operand (rows j), the site matrix S the B operand
+// (rows n), pre-split once per step by split_site_kernel into the shared-memory image of its
+// term planes.  Default tiles (cgemm_pair_kernel) are 256 rows j by Nt <= 128 columns n on a
+// pair of CTAs, with split accumulators in TMEM: hi x hi products go to "main" accumulators,
+// every cross-term product to "small" ones, added in the epilogue, so that the large
+// accumulators see two additions per k-step.  There the complex product is embedded in N: S is
+// held per term as planes Sr, Si, -Sr, and one MMA of N = 2 Nt takes Ar x [Sr; Si] into
 // (re, im) and another -Ai x [Si; -Sr], so each MMA reads A once for both halves.
-// QFX_TC_FAST_ACCUMULATION tiles are 128 x 256 with one accumulator pair
-// (re [0,256), im [256,512)) and four real products per term pair (4M).
-// Roles (14 warps):
-//   warps 0-3   producers: FP32 rows of B -> term planes in shared memory (K-major,
-//               no-swizzle core-matrix layout).  Default tiles take the rows from
-//               staging buffers filled by tensor-map copies (cp.async.bulk.tensor) when
-//               the shape allows it, otherwise they load them one k-stage ahead;
-//   warps 4-11  epilogue: TMEM -> registers -> C (two warps per TMEM lane quarter);
-//   warp 12     allocates TMEM; lane 0 issues tcgen05.mma;
-//   warp 13     lane 0 streams the pre-split image of S (written once per step by
-//               split_site_kernel in the same layout) with one bulk copy per stage;
-//               lane 1 issues the tensor-map copies of B.
+// QFX_TC_FAST_ACCUMULATION tiles (cgemm_fast_kernel) are 128 x 256 on one CTA with one
+// accumulator pair (re [0,256), im [256,512)) and four real products per term pair (4M).
+// Both kernels are persistent: producer warps split FP32 rows of B into term planes (K-major,
+// no-swizzle core-matrix layout), one thread issues the MMAs, others stream the site image with
+// bulk copies and, for pairs, the rows of B with tensor-map copies into staging buffers when
+// the shape allows it, and epilogue warps drain TMEM into C.
 // Rings of shared-memory stages are guarded by mbarriers.  Every wait has a deadline;
 // on expiry the kernel records an error, drains its own copies and MMAs, frees TMEM and
 // returns (the host reports QFX_ETIMEOUT).
@@ -41,8 +35,10 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 
+#include "launch.cuh"
 #include "ptx_async.cuh"
 #include "qfx_internal.h"
 
@@ -83,15 +79,17 @@ struct Mode<QFX_PREC_C3M_TF32X3> {
 };
 
 // ---- term splitting ------------------------------------------------------------
-// T BF16 terms of x: each the round-to-nearest of what the previous ones left
+// T BF16 terms of two numbers, packed (x0 in the low half): each the round-to-nearest of what
+// the previous ones left
 template <int T>
-__device__ __forceinline__ void split_bf16(float x, uint16_t t[T]) {
-  float r = x;
+__device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t t[T]) {
 #pragma unroll
   for (int i = 0; i < T; ++i) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(r);
-    t[i] = __bfloat16_as_ushort(h);
-    r -= __bfloat162float(h);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(t[i]) : "f"(x1), "f"(x0));
+    if (i + 1 < T) {
+      x0 -= __uint_as_float(t[i] << 16);
+      x1 -= __uint_as_float(t[i] & 0xffff0000u);
+    }
   }
 }
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -117,11 +115,10 @@ __device__ __forceinline__ void store_row_terms(char* plane0, int plane_bytes, i
     uint32_t w[T][8];
 #pragma unroll
     for (int k = 0; k < 16; k += 2) {
-      uint16_t a[T], b[T];
-      split_bf16<T>(x[k], a);
-      split_bf16<T>(x[k + 1], b);
+      uint32_t a[T];
+      split_bf16x2<T>(x[k], x[k + 1], a);
 #pragma unroll
-      for (int t = 0; t < T; ++t) w[t][k / 2] = (uint32_t)a[t] | ((uint32_t)b[t] << 16);
+      for (int t = 0; t < T; ++t) w[t][k / 2] = a[t];
     }
 #pragma unroll
     for (int t = 0; t < T; ++t) {
@@ -146,6 +143,25 @@ __device__ __forceinline__ void store_row_terms(char* plane0, int plane_bytes, i
     }
   }
   (void)sizeof(M_);
+}
+
+// One 16-byte half (kc) of a row's KS values as TERMS planes, for producers that share a row.
+template <int MODE>
+__device__ __forceinline__ void store_half_terms(char* plane0, int row, int kc, const float* x) {
+  constexpr int T = Mode<MODE>::TERMS;
+  char* pl = plane0 + (row >> 3) * 256 + kc * 128 + (row & 7) * 16;
+  uint32_t w[T][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint32_t t[T];
+    if constexpr (Mode<MODE>::FMT == 1) split_bf16x2<T>(x[2 * i], x[2 * i + 1], t);
+    else split_tf32x2(x[i], t);
+#pragma unroll
+    for (int q = 0; q < T; ++q) w[q][i] = t[q];
+  }
+#pragma unroll
+  for (int q = 0; q < T; ++q)
+    *reinterpret_cast<uint4*>(pl + q * kPlaneA) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
 }
 
 // ---- PTX helpers -----------------------------------------------------------------
@@ -182,7 +198,7 @@ __device__ __forceinline__ uint32_t instr_desc(int n, bool neg_a) {
 }
 template <int MODE>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  if constexpr (MODE == QFX_PREC_C3M_BF16X3) {
+  if constexpr (Mode<MODE>::FMT == 1) {
     asm volatile(
         "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
         "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
@@ -206,6 +222,71 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// ---- CTA pairs -------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// every thread of both CTAs, at points that each reaches (all waits before them are bounded)
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// Arrives on the barrier at this shared-memory offset in CTA 0 of the pair.  What it stands
+// for is ordered by itself (planes by the writers' proxy fences, TMEM reads by the tcgen05
+// fence), so the default scope is enough: a release at cluster scope waits for all of the
+// thread's stores, those of C among them, and made a k-stage take 2400 clk or more.
+__device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
+  asm volatile(
+      "{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, 0;\n"
+      "mbarrier.arrive.shared::cluster.b64 _, [r];\n}" ::"r"(bar) : "memory");
+}
+template <int MODE>
+__device__ __forceinline__ uint32_t instr_desc_pair(int n, bool neg_a) {   // M = 256 over both CTAs
+  return instr_desc<MODE>(n, neg_a) + ((uint32_t)(kRows >> 4) << 24);
+}
+template <int MODE>
+__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if constexpr (Mode<MODE>::FMT == 1) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+  } else {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+  }
+}
+// one arrival on the barrier at this offset in both CTAs once the MMAs issued so far are done
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3) : "memory");
+}
+
+// x / d and x % d in 32 bits where they hold it (a 64-bit division takes over a hundred clocks)
+__device__ __forceinline__ void divmod(int64_t x, int64_t d, int64_t& q, int64_t& r) {
+  if (((uint64_t)x | (uint64_t)d) >> 32) {
+    q = x / d;
+    r = x - q * d;
+  } else {
+    const uint32_t q32 = (uint32_t)x / (uint32_t)d;
+    q = q32;
+    r = (uint32_t)x - q32 * (uint32_t)d;
+  }
+}
+
 struct TcArgs {
   const float2* B; int64_t b_stride;
   float2* C; int64_t c_stride;
@@ -213,20 +294,17 @@ struct TcArgs {
   int64_t P, K, N, NL, Sd, J;
   int Nt;            // columns n per tile (<= 128 split accumulators, <= 256 single)
   int NHt;           // tiles along n per 128-row tile
-  int64_t JT;        // 128-row tiles per item
+  int64_t JT;        // 128-row tiles per item (256-row ones for pairs)
   int64_t tiles;     // total tiles (items x JT x NHt)
   int withhold_s;    // test hook: never stream S, so the bounded waits expire
-  int use_tma;       // producers read FP32 rows staged by tensor-map copies (default tiles)
+  int use_tma;       // pair tiles: producers read FP32 rows staged by tensor-map copies
+  int stages, nbuf;  // pair tiles: operand stages and staging buffers
   int box_s, box_p;  // tensor-map box: box_s consecutive s (columns), box_p values of p
   int beta;          // 1: add the product into C (a chunk of a long contraction)
 };
 
-// Persistent CTA, one per SM.  TMEM columns: with SPLITACC the hh-term products go to
-// "main" accumulators (re [0,Nt), im [Nt,2Nt)) and every cross-term product to "small"
-// ones (re [256,256+Nt), im [256+Nt,256+2Nt)), so the large accumulator sees 2 additions
-// per k-stage instead of 2 x NPROD; without SPLITACC re = [0, Nt), im = [256, 256 + Nt).
-// Warps: 0-3 producers, 4-11 epilogue (two per TMEM lane quarter, each half the columns),
-// 12 TMEM owner + MMA issuer, 13 S stream and tensor-map copies.
+// Operand stages start on 128-byte boundaries (tensor-map copies land there; the dynamic
+// window itself is only 16-byte aligned behind the static shared variables).
 constexpr uint32_t kAlignPad = 128;
 
 // Tile t -> (item g, 128-row tile jt, column tile nh).  Within an item the column tiles
@@ -237,55 +315,45 @@ constexpr uint32_t kAlignPad = 128;
 constexpr int64_t kBand = 8;
 __device__ __forceinline__ void tile_coords(const TcArgs& a, int64_t t, int64_t& g, int64_t& jt,
                                             int64_t& nh) {
-  const int64_t per_item = a.JT * a.NHt;
-  g = t / per_item;
-  int64_t r = t - g * per_item;
-  const int64_t band = r / (kBand * a.JT);
+  int64_t r, band;
+  divmod(t, a.JT * a.NHt, g, r);
+  divmod(r, kBand * a.JT, band, r);
   const int64_t n0 = band * kBand;
   const int64_t w = a.NHt - n0 < kBand ? a.NHt - n0 : kBand;
-  r -= band * kBand * a.JT;
-  jt = r / w;
-  nh = n0 + (r - jt * w);
+  divmod(r, w, jt, r);
+  nh = n0 + r;
 }
 
-template <int MODE, bool SPLITACC>
-struct TcCfg {
+// ---- fast accumulation: one CTA per SM, one accumulator pair -------------------------
+// re in TMEM columns [0, Nt), im in [256, 256 + Nt).  Warps: 0-3 producers, 4-11 epilogue (two
+// per TMEM lane quarter, each half the columns), 12 TMEM owner + MMA issuer, 13 site stream.
+template <int MODE>
+struct FastCfg {
   using M_ = Mode<MODE>;
-  static constexpr int NT_MAX = SPLITACC ? 128 : 256;
-  // default tiles hold S as [Sr; Si; -Sr] per term (the complex product embedded in N)
-  static constexpr int PLANES = 2 * M_::TERMS;             // A planes per stage
-  static constexpr int SPLANES = SPLITACC ? 3 * M_::TERMS : PLANES;   // S planes per stage
-  static constexpr int STAGES = SPLITACC ? (M_::TERMS == 3 ? 3 : 4) : 3;
+  static constexpr int NT_MAX = 256;
+  static constexpr int PLANES = 2 * M_::TERMS;             // planes of each operand per stage
+  static constexpr int STAGES = 3;
   static constexpr int STAGE_A = PLANES * kPlaneA;
   static constexpr int THREADS = 14 * 32;
-  // FP32 rows of the default tile arrive by tensor-map copies into NBUF staging buffers;
-  // the fast tile's operand ring leaves no room and keeps register prefetch
-  static constexpr int STAGE_IN = kRows * M_::KS * 8;
-  static constexpr int NBUF = SPLITACC ? (M_::KS == 16 ? 2 : 4) : 0;
   static size_t smem(int nt) {
-    return kAlignPad + (size_t)STAGES * (STAGE_A + SPLANES * nt * 32) + (size_t)NBUF * STAGE_IN +
-           (3 * STAGES + 3 + 2 * NBUF) * sizeof(uint64_t);
+    return kAlignPad + (size_t)STAGES * (STAGE_A + PLANES * nt * 32) + (3 * STAGES + 3) * sizeof(uint64_t);
   }
 };
 
-template <int MODE, bool SPLITACC>
-__global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
-    cgemm_tc_kernel(const TcArgs a, const __grid_constant__ CUtensorMap tmA) {
+template <int MODE>
+__global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(const TcArgs a) {
   using M_ = Mode<MODE>;
-  using CF = TcCfg<MODE, SPLITACC>;
+  using CF = FastCfg<MODE>;
   constexpr int TERMS = M_::TERMS, KS = M_::KS, STAGES = CF::STAGES;
   extern __shared__ __align__(16) char smem_raw[];
-  // tensor-map copies land on 128-byte boundaries; the dynamic window itself is only
-  // 16-byte aligned behind the static shared variables
   char* smem = smem_raw + ((kAlignPad - (smem_u32(smem_raw) & (kAlignPad - 1))) & (kAlignPad - 1));
   const int stageA = CF::STAGE_A;
   const int planeS = a.Nt * 32;
-  const int stageS = CF::SPLANES * planeS;
+  const int stageS = CF::PLANES * planeS;
   char* sA = smem;
   char* sS = smem + STAGES * stageA;
-  char* sIn = sS + STAGES * stageS;                 // NBUF x [box_p][KS][box_s] float2
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sIn + CF::NBUF * CF::STAGE_IN);
-  // bars: fullA[S], fullS[S], empty[S], acc_full, tmem_free, done, in_full[NBUF], in_empty[NBUF]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sS + STAGES * stageS);
+  // bars: fullA[S], fullS[S], empty[S], acc_full, tmem_free, done
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -297,8 +365,6 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
   const uint32_t acc_full = smem_u32(&bars[3 * STAGES]);
   const uint32_t tmem_free = smem_u32(&bars[3 * STAGES + 1]);
   const uint32_t done = smem_u32(&bars[3 * STAGES + 2]);
-  auto in_full = [&](int b) { return smem_u32(&bars[3 * STAGES + 3 + b]); };
-  auto in_empty = [&](int b) { return smem_u32(&bars[3 * STAGES + 3 + CF::NBUF + b]); };
 
   if (tid == 0) {
     abort_flag = 0;
@@ -310,10 +376,6 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
     mbar_init(acc_full, 1);
     mbar_init(tmem_free, 8);
     mbar_init(done, 1);
-    for (int b = 0; b < CF::NBUF; ++b) {
-      mbar_init(in_full(b), 1);
-      mbar_init(in_empty(b), kRows);
-    }
     mbar_init_fence();
   }
   if (warp == 12) {
@@ -329,39 +391,9 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
 
   if (warp < 4) {
     // ---- producers: split 128 rows of B per k-stage into term planes -------------------
-    // Rows arrive either through tensor-map copies staged NBUF k-stages ahead (default
-    // tiles, issued by warp 13) or through loads issued one k-stage ahead into registers,
-    // so their latency overlaps the split and the wait for a free operand stage.
+    // Rows are loaded one k-stage ahead into registers, so that their latency overlaps the
+    // split and the wait for a free operand stage.
     int64_t t = blockIdx.x, it = 0, q = 0;
-    if (CF::NBUF > 0 && a.use_tma) {
-      const int ps = tid / a.box_s, ss = tid % a.box_s;     // this row inside the box
-      while (t < a.tiles && !*abort) {
-        const int b = (int)(q % (CF::NBUF > 0 ? CF::NBUF : 1));
-        if (!mbar_wait(in_full(b), (uint32_t)((q / (CF::NBUF > 0 ? CF::NBUF : 1)) & 1), abort)) break;
-        const float2* in = reinterpret_cast<const float2*>(sIn + b * CF::STAGE_IN);
-        float re[KS], im[KS];
-#pragma unroll
-        for (int kk = 0; kk < KS; ++kk) {
-          const float2 v = in[(ps * KS + kk) * a.box_s + ss];
-          re[kk] = v.x;
-          im[kk] = v.y;
-        }
-        // the next tensor-map copy rewrites this buffer through the async proxy: order
-        // these generic reads before it (without the fence, fast consumers saw rows of the
-        // following k-stage)
-        fence_async_smem();
-        mbar_arrive(in_empty(b));
-        const int s = (int)(q % STAGES);
-        if (q >= STAGES && !mbar_wait(empty(s), (uint32_t)((q / STAGES - 1) & 1), abort)) break;
-        char* st = sA + s * stageA;
-        store_row_terms<MODE>(st, kPlaneA, tid, re);
-        store_row_terms<MODE>(st + TERMS * kPlaneA, kPlaneA, tid, im);
-        fence_async_smem();
-        mbar_arrive(fullA(s));
-        ++q;
-        if (++it == KT) { it = 0; t += gridDim.x; }
-      }
-    } else {
     auto row_ptr = [&](int64_t tt, int64_t& pofs) -> const float2* {
       int64_t g, jt, nh;
       tile_coords(a, tt, g, jt, nh);
@@ -396,7 +428,6 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
       t = nt;
       it = ni;
     }
-    }
   } else if (warp == 13) {
     // ---- S image stream ------------------------------------------------------------
     if (lane == 0) {
@@ -421,39 +452,13 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
         while (!mbar_try(fullS(s), (uint32_t)((i / STAGES) & 1)) && globaltimer() < deadline) {
         }
       }
-    } else if (lane == 1 && CF::NBUF > 0 && a.use_tma) {
-      // ---- FP32 rows of B: one tensor-map copy per (tile, k-stage) into staging --------
-      constexpr int NB = CF::NBUF > 0 ? CF::NBUF : 1;
-      int64_t q = 0, issued = 0;
-      bool ok = true;
-      for (int64_t t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
-        int64_t g, jt, nh;
-        tile_coords(a, t, g, jt, nh);
-        const int64_t j0 = jt * kRows;
-        const int c0 = (int)(j0 % a.Sd), c2 = (int)(j0 / a.Sd);
-        for (int64_t it = 0; it < KT; ++it, ++q) {
-          const int b = (int)(q % NB);
-          if (q >= NB && !mbar_wait(in_empty(b), (uint32_t)((q / NB - 1) & 1), abort, 32)) { ok = false; break; }
-          mbar_arrive_tx(in_full(b), (uint32_t)CF::STAGE_IN);
-          tma_load_4d(smem_u32(sIn + b * CF::STAGE_IN), &tmA, c0, (int)(it * KS), c2, (int)g, in_full(b));
-          issued = q + 1;
-        }
-      }
-      for (int64_t i = (issued > NB ? issued - NB : 0); i < issued; ++i) {
-        const int b = (int)(i % NB);
-        const unsigned long long deadline = globaltimer() + kWaitNs;
-        while (!mbar_try(in_full(b), (uint32_t)((i / NB) & 1)) && globaltimer() < deadline) {
-        }
-      }
     }
   } else if (warp == 12) {
     // ---- MMA issue -----------------------------------------------------------------
     if (lane == 0) {
       int64_t q = 0, tc = 0;
       bool ok = true;
-      // default tiles: one MMA covers re and im (N = 2 Nt); fast tiles: N = Nt
-      const int n_mma = SPLITACC ? 2 * a.Nt : a.Nt;
-      const uint32_t idesc_p = instr_desc<MODE>(n_mma, false), idesc_n = instr_desc<MODE>(n_mma, true);
+      const uint32_t idesc_p = instr_desc<MODE>(a.Nt, false), idesc_n = instr_desc<MODE>(a.Nt, true);
       for (int64_t t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tc) {
         if (tc > 0 && !mbar_wait(tmem_free, (uint32_t)((tc - 1) & 1), abort)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -464,22 +469,7 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
           if (!mbar_wait(fullA(s), par, abort) || !mbar_wait(fullS(s), par, abort)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a0 = smem_u32(sA + s * stageA), b0 = smem_u32(sS + s * stageS);
-          if constexpr (SPLITACC) {
-            // Ar x [Sr; Si] -> (re, im) += (Ar Sr, Ar Si);  (-Ai) x [Si; -Sr] -> += (-Ai Si, Ai Sr)
-#pragma unroll
-            for (int ca = 0; ca < 2; ++ca) {
-#pragma unroll
-              for (int pi = 0; pi < M_::NPROD; ++pi) {
-                const bool main_term = M_::ta(pi) == 0 && M_::tb(pi) == 0;
-                const int acc = main_term ? 0 : 1;
-                const uint64_t ad = smem_desc(a0 + (ca * TERMS + M_::ta(pi)) * kPlaneA);
-                const uint64_t bd = smem_desc(b0 + (3 * M_::tb(pi) + ca) * planeS);
-                mma<MODE>(tmem + (uint32_t)(acc * 256), ad, bd, ca ? idesc_n : idesc_p, started[acc] ? 1u : 0u);
-                started[acc] = true;
-              }
-            }
-          } else {
-            // 4M with re in TMEM columns [0, Nt) and im in [256, 256 + Nt)
+          {   // 4M with re in TMEM columns [0, Nt) and im in [256, 256 + Nt)
 #pragma unroll
             for (int rp = 0; rp < 4; ++rp) {
               const int ca = (rp == 0 || rp == 2) ? 0 : 1;          // Ar, Ai, Ar, Ai
@@ -530,21 +520,9 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
       for (int ci = half; ci < nchunks; ci += 2) {
         const int c0 = ci * 16;
         float vr[16], vi[16];
-        if (SPLITACC) {
-          // main (re, im) in columns [0, Nt), [Nt, 2 Nt); small ones 256 further
-          float sr[16], si[16];
-          tmem_ld16(tmem + lane_base + c0, vr);
-          tmem_ld16(tmem + lane_base + a.Nt + c0, vi);
-          tmem_ld16(tmem + lane_base + 256 + c0, sr);
-          tmem_ld16(tmem + lane_base + 256 + a.Nt + c0, si);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int i = 0; i < 16; ++i) { vr[i] += sr[i]; vi[i] += si[i]; }
-        } else {
-          tmem_ld16(tmem + lane_base + c0, vr);
-          tmem_ld16(tmem + lane_base + 256 + c0, vi);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        }
+        tmem_ld16(tmem + lane_base + c0, vr);
+        tmem_ld16(tmem + lane_base + 256 + c0, vi);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if (ci == my_last) {
           // last TMEM read of this tile by this warp: hand the columns back to the MMA
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -597,6 +575,434 @@ __global__ void __launch_bounds__(TcCfg<MODE, SPLITACC>::THREADS, 1)
   }
 }
 
+// ---- default tiles on CTA pairs ------------------------------------------------------
+// Two CTAs of a cluster (the two SMs of a TPC) compute 256 rows j x Nt columns n together:
+// one tcgen05.mma.cta_group::2 of M = 256 takes 128 rows of B from each CTA and half of the
+// 2 Nt rows of the embedded site operand from each, so an SM's shared memory holds and feeds
+// its tensor core half of that operand (Sr and Si in CTA 0, Si and -Sr in CTA 1), where a
+// CTA by itself reads all of it for every MMA.  Per BF16x3 k-step and SM at Nt = 128 that is
+//   MMA reads 12 x (4 + 4) KB, site stream 24 KB, term planes 24 KB, staging 2 x 16 KB:
+//   176 KB = 1375 clk at 128 B/clk against 1638 clk of MMA at the measured rate,
+// where a single CTA moves 236 KB = 1844 clk.  Measured against such a single CTA (K = N = 256,
+// 2^19 columns): one cool launch takes 0.82 ms (0.83 of the tensor probe) against 0.98; run
+// for seconds both are held by the 1400 W limit, 1.02 against 1.07 ms for BF16x3 and 0.97
+// against 1.02 for TF32x3; BF16x2 at K = N = 1024 over 2^15 columns went from 0.67 to 0.53 ms.
+//
+// With 4 Nt <= 256 the accumulators of two tiles fit the TMEM (the halves of its 512
+// columns): the MMAs of a tile run while the epilogue stores the one before.  At Nt = 128
+// they take turns, and the MMAs wait until the epilogue has read them.  Its stores back up
+// (100 clk for each of 256 bytes, with every SM storing at once), so it reads ahead of them:
+// with registers taken over from the other roles it holds 6 chunks of 8 columns beside the one
+// it stores, and hands the TMEM back after the second of its 8 chunks.
+//
+// Roles, in each CTA on its own 128 rows: warps 0-7 producers, 8 TMEM owner and MMA issuer, 9
+// site stream, 10 tensor-map copies, 12-19 epilogue (two per TMEM lane quarter).  CTA 0 (the
+// leader) issues every MMA; its barriers collect the arrivals of both CTAs, and the commits
+// arrive on the barriers of both.  Warp 8 of CTA 1 passes the arrival of its site copies on to
+// the leader.
+// A CTA leaves only after the cluster barrier at the end, when nothing refers to it any more.
+template <int MODE>
+struct PairCfg {
+  using M_ = Mode<MODE>;
+  static constexpr int NT_MAX = 128;
+  // k-steps (of one MMA per product) in an operand stage: the fences, arrivals and waits of a
+  // stage cost its roles 500 to 800 clk, which the 6 MMAs of a two-term k-step (819 clk) barely
+  // cover.  Two k-steps of TF32 take the bytes of one of BF16 (K = N = 256 over 2^19 columns:
+  // 984 -> 903 us); two of BF16x2 leave room for two stages only (490 -> 515 us at K = 1024).
+  static constexpr int SUB = M_::KS == 8 ? 2 : 1;
+  static constexpr int PLANES = 2 * M_::TERMS;              // planes of each operand per k-step
+  static constexpr int STAGE_A = SUB * PLANES * kPlaneA;
+  static constexpr int STAGE_IN = kRows * SUB * M_::KS * 8;
+  static constexpr int MAX_STAGES = 8, MAX_BUF = 8;
+  static constexpr int NBARS = 3 * MAX_STAGES + 5 + 2 * MAX_BUF;
+  static constexpr int THREADS = 20 * 32;
+  static size_t smem(int nt, int stages, int nbuf) {
+    return kAlignPad + (size_t)stages * (STAGE_A + SUB * PLANES * nt * 32) + (size_t)nbuf * STAGE_IN +
+           NBARS * sizeof(uint64_t);
+  }
+};
+
+// Position in a ring of `n` slots and the parity of its current pass.
+struct Ring {
+  int i = 0;
+  uint32_t pass = 0;
+  __device__ __forceinline__ void step(int n) {
+    if (++i == n) { i = 0; pass ^= 1u; }
+  }
+};
+template <int N>
+__device__ __forceinline__ void reg_release() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_take() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+// Registers per thread of the roles' warpgroups; the launch gives each of the five 96.
+constexpr int kRegLaunch = 96, kRegProd = 72, kRegCtl = 48, kRegEpi = 144;
+static_assert(2 * kRegProd + kRegCtl + 2 * kRegEpi <= 5 * kRegLaunch, "the roles share the launch's registers");
+
+template <int MODE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREADS, 1)
+    cgemm_pair_kernel(const TcArgs a, const __grid_constant__ CUtensorMap tmA) {
+  using M_ = Mode<MODE>;
+  using CF = PairCfg<MODE>;
+  constexpr int TERMS = M_::TERMS, KS = M_::KS, SUB = CF::SUB;
+  extern __shared__ __align__(16) char smem_raw[];
+  char* smem = smem_raw + ((kAlignPad - (smem_u32(smem_raw) & (kAlignPad - 1))) & (kAlignPad - 1));
+  const int planeS = a.Nt * 32;
+  const int stepS = CF::PLANES * planeS, stageS = SUB * stepS;
+  const int stages = a.stages, nbuf = a.nbuf;
+  char* sA = smem;
+  char* sS = smem + stages * CF::STAGE_A;
+  char* sIn = sS + stages * stageS;                 // nbuf x [box_p][SUB * KS][box_s] float2
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sIn + nbuf * CF::STAGE_IN);
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ int abort_flag;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_rank();
+  const int k_steps = (int)(a.K / KS);                // the last stage of a tile may have fewer
+  const int KT = (k_steps + SUB - 1) / SUB;
+  const int n_acc = 4 * a.Nt <= 256 ? 2 : 1;         // tiles whose accumulators fit the TMEM
+
+  const uint32_t bar0 = smem_u32(bars);
+  auto full = [&](int s) { return bar0 + 8 * s; };                         // leader's: stage s of both CTAs
+  auto fullS = [&](int s) { return bar0 + 8 * (CF::MAX_STAGES + s); };     // CTA 1's: its site copies
+  auto empty = [&](int s) { return bar0 + 8 * (2 * CF::MAX_STAGES + s); };
+  auto acc_full = [&](int c) { return bar0 + 8 * (3 * CF::MAX_STAGES + c); };
+  auto tmem_free = [&](int c) { return bar0 + 8 * (3 * CF::MAX_STAGES + 2 + c); };   // leader's: both epilogues
+  const uint32_t done = bar0 + 8 * (3 * CF::MAX_STAGES + 4);
+  auto in_full = [&](int b) { return bar0 + 8 * (3 * CF::MAX_STAGES + 5 + b); };
+  auto in_empty = [&](int b) { return bar0 + 8 * (3 * CF::MAX_STAGES + 5 + CF::MAX_BUF + b); };
+
+  if (tid == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full(s), 18);        // 8 producer warps and the site copies of each CTA
+      mbar_init(fullS(s), 1);
+      mbar_init(empty(s), 1);
+    }
+    for (int c = 0; c < 2; ++c) {
+      mbar_init(acc_full(c), 1);
+      mbar_init(tmem_free(c), 16);   // 8 epilogue warps of each CTA
+    }
+    mbar_init(done, 1);
+    for (int b = 0; b < nbuf; ++b) {
+      mbar_init(in_full(b), 1);
+      mbar_init(in_empty(b), 8);
+    }
+    mbar_init_fence();
+  }
+  __syncwarp();
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_base_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_barrier();   // barriers of both CTAs initialised, TMEM allocated in both
+  launch_wait();       // the site image is written
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base_slot;
+  volatile int* abort = &abort_flag;
+  const int64_t pair0 = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  // tile t of the pair: a.JT counts 256-row tiles, this CTA has rows [128 jt, 128 jt + 128)
+  auto coords = [&](int64_t t, int64_t& g, int64_t& jt, int64_t& nh) {
+    tile_coords(a, t, g, jt, nh);
+    jt = 2 * jt + rank;
+  };
+
+  if (warp < 8) {
+    // ---- producers: split 128 rows of B per k-stage into term planes -------------------
+    reg_release<kRegProd>();
+    // Two threads share a row, each half of its k.  The proxy fence is the largest part of a
+    // stage's latency, so there is one for both what it orders: the operand planes before the
+    // MMAs that read them, and the reads of the staging buffer before the copy that reuses it.
+    constexpr int KH = KS / 2;
+    const int prow = tid & (kRows - 1), kh = tid >> 7;
+    const int64_t n_stages = pair0 < a.tiles ? ((a.tiles - pair0 + pairs - 1) / pairs) * KT : 0;
+    Ring op;                    // operand stages
+    float re[SUB][KH], im[SUB][KH];
+    auto put = [&]() -> bool {   // re, im into the next operand stage; false on a timeout
+      if (!__all_sync(0xffffffffu, mbar_wait(empty(op.i), op.pass ^ 1u, abort))) return false;
+      char* st = sA + op.i * CF::STAGE_A;
+#pragma unroll
+      for (int u = 0; u < SUB; ++u) {
+        store_half_terms<MODE>(st + u * CF::PLANES * kPlaneA, prow, kh, re[u]);
+        store_half_terms<MODE>(st + (u * CF::PLANES + TERMS) * kPlaneA, prow, kh, im[u]);
+      }
+      fence_async_smem();
+      __syncwarp();
+      return true;
+    };
+    if (a.use_tma) {
+      const int ps = prow / a.box_s, ss = prow % a.box_s;     // this row inside the box
+      const int in_ofs = (ps * SUB * KS + kh * KH) * a.box_s + ss;
+      Ring in;
+      for (int64_t q = 0; q < n_stages; ++q) {
+        if (!__all_sync(0xffffffffu, mbar_wait(in_full(in.i), in.pass, abort))) break;
+        const float2* src = reinterpret_cast<const float2*>(sIn + in.i * CF::STAGE_IN) + in_ofs;
+#pragma unroll
+        for (int u = 0; u < SUB; ++u)
+#pragma unroll
+          for (int kk = 0; kk < KH; ++kk) {   // rows past K arrive as zeros
+            const float2 v = src[(u * KS + kk) * a.box_s];
+            re[u][kk] = v.x;
+            im[u][kk] = v.y;
+          }
+        if (!put()) break;
+        if (lane == 0) {
+          mbar_arrive_leader(full(op.i));
+          mbar_arrive(in_empty(in.i));
+        }
+        op.step(stages);
+        in.step(nbuf);
+      }
+    } else {
+      // rows that no tensor map describes: loads issued one k-stage ahead into registers
+      float2 nxt[SUB][KH];
+      int64_t t = pair0;
+      int it = 0;
+      bool inside = false;
+      const float2* src = nullptr;
+      auto fetch = [&]() {
+        if (it == 0) {
+          int64_t g, jt, nh, p, sidx;
+          coords(t, g, jt, nh);
+          const int64_t jg = jt * kRows + prow;
+          inside = jg < a.J;
+          divmod(jg, a.Sd, p, sidx);
+          src = a.B + g * a.b_stride + p * a.K * a.Sd + sidx + (int64_t)(kh * KH) * a.Sd;
+        }
+#pragma unroll
+        for (int u = 0; u < SUB; ++u)
+#pragma unroll
+          for (int kk = 0; kk < KH; ++kk)
+            nxt[u][kk] = inside && it * SUB + u < k_steps ? __ldg(src + (u * KS + kk) * a.Sd) : make_float2(0.f, 0.f);
+        src += SUB * KS * a.Sd;
+        if (++it == KT) { it = 0; t += pairs; }
+      };
+      if (n_stages > 0) fetch();
+      for (int64_t q = 0; q < n_stages; ++q) {
+#pragma unroll
+        for (int u = 0; u < SUB; ++u)
+#pragma unroll
+          for (int kk = 0; kk < KH; ++kk) { re[u][kk] = nxt[u][kk].x; im[u][kk] = nxt[u][kk].y; }
+        if (q + 1 < n_stages) fetch();
+        if (!put()) break;
+        if (lane == 0) mbar_arrive_leader(full(op.i));
+        op.step(stages);
+      }
+    }
+  } else if (warp < 12) {
+    reg_release<kRegCtl>();
+    if (warp == 9 && lane == 0) {
+      // ---- site image stream: per term the two planes of this CTA's half ---------------
+      Ring st;
+      int64_t issued = 0;
+      bool ok = !a.withhold_s;
+      for (int64_t t = pair0; t < a.tiles && ok; t += pairs) {
+        int64_t g, jt, nh;
+        coords(t, g, jt, nh);
+        const char* src = a.simage + g * a.img_stride + nh * (3 * TERMS) * planeS + rank * planeS;
+        for (int it = 0; it < KT; ++it) {
+          if (!mbar_wait(empty(st.i), st.pass ^ 1u, abort)) { ok = false; break; }
+          const uint32_t bar = rank == 0 ? full(st.i) : fullS(st.i);
+          const int subs = k_steps - it * SUB < SUB ? k_steps - it * SUB : SUB;
+          mbar_arrive_tx(bar, (uint32_t)(subs * stepS));
+          for (int u = 0; u < subs; ++u) {
+#pragma unroll
+            for (int tm = 0; tm < TERMS; ++tm)
+              bulk_copy(smem_u32(sS + st.i * stageS + u * stepS + tm * 2 * planeS), src + (int64_t)tm * 3 * planeS,
+                        (uint32_t)(2 * planeS), bar);
+            src += (int64_t)a.NHt * (3 * TERMS) * planeS;
+          }
+          st.step(stages);
+          ++issued;
+        }
+      }
+      // every issued copy must land before the CTA exits: the MMAs that the leader waits for
+      // at the end read all of them, but after a timeout they may be in flight, so their
+      // barriers are watched here (a limit for each, as everywhere)
+      if (*abort) {
+        for (int64_t i = 0; i < (issued < stages ? issued : stages); ++i) {
+          st.i = st.i == 0 ? stages - 1 : st.i - 1;
+          if (st.i == stages - 1) st.pass ^= 1u;
+          const uint32_t bar = rank == 0 ? full(st.i) : fullS(st.i);
+          const unsigned long long deadline = globaltimer() + kWaitNs / 100;
+          while (!mbar_try(bar, st.pass) && globaltimer() < deadline) {
+          }
+        }
+      }
+    } else if (warp == 10 && lane == 0 && a.use_tma) {
+      // ---- FP32 rows of B: one tensor-map copy per (tile, k-stage) into staging --------
+      Ring in;
+      int64_t issued = 0;
+      bool ok = true;
+      for (int64_t t = pair0; t < a.tiles && ok; t += pairs) {
+        int64_t g, jt, nh, p, sidx;
+        coords(t, g, jt, nh);
+        divmod(jt * kRows, a.Sd, p, sidx);
+        for (int it = 0; it < KT; ++it) {
+          if (!mbar_wait(in_empty(in.i), in.pass ^ 1u, abort)) { ok = false; break; }
+          mbar_arrive_tx(in_full(in.i), (uint32_t)CF::STAGE_IN);
+          tma_load_4d(smem_u32(sIn + in.i * CF::STAGE_IN), &tmA, (int)sidx, it * SUB * KS, (int)p, (int)g, in_full(in.i));
+          in.step(nbuf);
+          ++issued;
+        }
+      }
+      for (int64_t i = 0; i < (issued < nbuf ? issued : nbuf); ++i) {   // newest first
+        in.i = in.i == 0 ? nbuf - 1 : in.i - 1;
+        if (in.i == nbuf - 1) in.pass ^= 1u;
+        const unsigned long long deadline = globaltimer() + kWaitNs;
+        while (!mbar_try(in_full(in.i), in.pass) && globaltimer() < deadline) {
+        }
+      }
+    } else if (warp == 8 && lane == 0 && rank == 0) {
+      // ---- MMA issue -------------------------------------------------------------------
+      Ring st, acc;
+      bool ok = true;
+      const uint32_t idesc_p = instr_desc_pair<MODE>(2 * a.Nt, false), idesc_n = instr_desc_pair<MODE>(2 * a.Nt, true);
+      const uint32_t small = (uint32_t)(n_acc == 2 ? 2 * a.Nt : 256);
+      for (int64_t t = pair0; t < a.tiles && ok; t += pairs) {
+        if (!mbar_wait(tmem_free(acc.i), acc.pass ^ 1u, abort)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d0 = tmem + (uint32_t)(acc.i * 256);
+        bool started[2] = {false, false};
+        for (int it = 0; it < KT; ++it) {
+          if (!mbar_wait(full(st.i), st.pass, abort)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+          for (int u = 0; u < SUB; ++u) {
+            if (u > 0 && it * SUB + u >= k_steps) break;
+            const uint32_t a0 = smem_u32(sA + st.i * CF::STAGE_A) + u * CF::PLANES * kPlaneA;
+            const uint32_t b0 = smem_u32(sS + st.i * stageS) + u * stepS;
+            // Ar x [Sr; Si] -> (re, im) += (Ar Sr, Ar Si);  (-Ai) x [Si; -Sr] -> += (-Ai Si, Ai Sr)
+#pragma unroll
+            for (int ca = 0; ca < 2; ++ca) {
+#pragma unroll
+              for (int pi = 0; pi < M_::NPROD; ++pi) {
+                const int k = M_::ta(pi) == 0 && M_::tb(pi) == 0 ? 0 : 1;   // hi x hi products: main
+                const uint64_t ad = smem_desc(a0 + (ca * TERMS + M_::ta(pi)) * kPlaneA);
+                const uint64_t bd = smem_desc(b0 + (2 * M_::tb(pi) + ca) * planeS);
+                mma_pair<MODE>(d0 + (k ? small : 0u), ad, bd, ca ? idesc_n : idesc_p, started[k] ? 1u : 0u);
+                started[k] = true;
+              }
+            }
+          }
+          mma_commit_pair(empty(st.i));
+          st.step(stages);
+        }
+        if (ok) mma_commit_pair(acc_full(acc.i));
+        acc.step(n_acc);
+      }
+      mma_commit_pair(done);
+    } else if (warp == 8 && lane == 0) {
+      // ---- CTA 1: its site copies have landed ------------------------------------------
+      Ring st;
+      bool ok = true;
+      for (int64_t t = pair0; t < a.tiles && ok; t += pairs)
+        for (int it = 0; it < KT; ++it) {
+          if (!mbar_wait(fullS(st.i), st.pass, abort)) { ok = false; break; }
+          mbar_arrive_leader(full(st.i));
+          st.step(stages);
+        }
+    }
+    __syncwarp();
+  } else {
+    // ---- epilogue: TMEM -> C -----------------------------------------------------------
+    reg_take<kRegEpi>();
+    const int quarter = warp & 3, half = (warp - 12) >> 2;
+    const int row = quarter * 32 + lane;
+    const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+    // 8-column chunks alternate between the two warps of a lane quarter: chunks half, half + 2,
+    // ..., AHEAD of them in registers before the first is stored
+    constexpr int MOST = CF::NT_MAX / 16, AHEAD = 5, RING = AHEAD + 1;
+    const int mine = a.Nt / 16;
+    const int NL = (int)a.NL;
+    const int64_t wrap = a.P * a.NL * a.Sd - (int64_t)NL * a.Sd;   // from the end of one nh to the next
+    Ring acc;
+    for (int64_t t = pair0; t < a.tiles; t += pairs) {
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full(acc.i), acc.pass, abort, 64))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t main0 = tmem + (uint32_t)(acc.i * 256) + lane_base;
+      const uint32_t small0 = main0 + (uint32_t)(n_acc == 2 ? 2 * a.Nt : 256);
+      float vr[RING][8], vi[RING][8];
+      auto load = [&](int i, int buf) {   // main + small of this warp's chunk i
+        const uint32_t c0 = (uint32_t)((half + 2 * i) * 8);
+        float sr[8], si[8];
+        tmem_ld8(main0 + c0, vr[buf]);
+        tmem_ld8(main0 + a.Nt + c0, vi[buf]);
+        tmem_ld8(small0 + c0, sr);
+        tmem_ld8(small0 + a.Nt + c0, si);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { vr[buf][e] += sr[e]; vi[buf][e] += si[e]; }
+        if (i + 1 == mine) {   // this warp has read the accumulators: back to the MMAs
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive_leader(tmem_free(acc.i));
+        }
+      };
+#pragma unroll
+      for (int i = 0; i < AHEAD; ++i)
+        if (i < mine) load(i, i);
+      int64_t g, jt, nh, p, sidx;
+      coords(t, g, jt, nh);
+      const int64_t jg = jt * kRows + row;
+      const bool valid = jg < a.J;
+      divmod(jg, a.Sd, p, sidx);
+      float2* Cj = a.C + g * a.c_stride + p * a.NL * a.Sd + sidx;
+#pragma unroll
+      for (int i = 0; i < MOST; ++i) {
+        if (i + AHEAD < MOST && i + AHEAD < mine) load(i + AHEAD, (i + AHEAD) % RING);
+        if (i < mine && valid) {
+          const int buf = i % RING;
+          // one division per chunk, then step along n with a carry into nh
+          const int n0 = (int)nh * a.Nt + (half + 2 * i) * 8;
+          const int nh0 = n0 / NL;
+          int left = (nh0 + 1) * NL - n0;   // columns to the end of this nh
+          float2* dst = Cj + nh0 * wrap + (int64_t)n0 * a.Sd;
+          if (a.beta) {   // a chunk of a long contraction: add into C
+            // all 8 reads first (C is written only by this tile in this launch, so the
+            // read-only path applies): one memory latency per chunk, not one per element
+            float2 o[8];
+            const float2* d = dst;
+            int l = left;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              o[e] = __ldg(d);
+              d += a.Sd;
+              if (--l == 0) { l = NL; d += wrap; }
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { vr[buf][e] += o[e].x; vi[buf][e] += o[e].y; }
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            *dst = make_float2(vr[buf][e], vi[buf][e]);
+            dst += a.Sd;
+            if (--left == 0) { left = NL; dst += wrap; }
+          }
+        }
+      }
+      acc.step(n_acc);
+    }
+  }
+
+  __syncwarp();
+  if (warp == 8) mbar_wait(done, 0, abort, 256);   // last MMAs finished before freeing TMEM
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_barrier();
+  if (warp == 8) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  }
+  cluster_barrier();   // neither CTA leaves while the other still frees its half
+}
+
 // Pre-split of the site matrix S[k][n] into the per-stage shared-memory image, per
 // (stage ks, n tile), each plane [row n within the tile][32 bytes]:
 //   EMB (default tiles): per term t the planes Sr_t, Si_t, -Sr_t, so that [Sr_t; Si_t]
@@ -608,6 +1014,7 @@ __global__ void __launch_bounds__(128) split_site_kernel(const float2* __restric
                                                           int64_t img_stride) {
   using M_ = Mode<MODE>;
   constexpr int TERMS = M_::TERMS, KS = M_::KS;
+  launch_next();
   const int n = blockIdx.x * 128 + threadIdx.x;
   const int ks = blockIdx.y;
   const int g = blockIdx.z;
@@ -638,8 +1045,8 @@ __global__ void __launch_bounds__(128) split_site_kernel(const float2* __restric
   }
 }
 
-// Tensor map over B viewed as (s, k, p, item) 8-byte elements, box (box_s, KS, box_p, 1)
-// = one 128-row, KS-deep k-stage of a tile.  False if the shape does not allow it (the
+// Tensor map over B viewed as (s, k, p, item) 8-byte elements, box (box_s, ks, box_p, 1)
+// = one 128-row, ks-deep k-stage of a tile.  False if the shape does not allow it (the
 // box's inner extent must be at least 16 bytes: Sd >= 2; tiles must not straddle p
 // unevenly: Sd a multiple of 128 or a divisor of it).
 bool make_b_map(CUtensorMap* map, const void* B, int64_t b_stride, int batch, int64_t P, int64_t K,
@@ -662,35 +1069,54 @@ bool make_b_map(CUtensorMap* map, const void* B, int64_t b_stride, int batch, in
   return true;
 }
 
-// Shared-memory opt-in of one tensor-core kernel, once per device (also called ahead of a
-// graph capture).
-template <int MODE, bool SPLITACC>
+// Staging buffers (16 KB each) of a pair tile, and as many operand stages as the rest of the
+// shared memory holds: 3 buffers, but 2 for TF32, whose 64 KB stages then number 3 at Nt = 128
+// instead of 2 (K = N = 256 over 2^19 columns: 903 us against 946; BF16x3 927 with 2 buffers and
+// 926 with 3, at K = N = 64 over 2^21 columns 446 and 433).
+constexpr int kMaxSmem = 227 << 10;   // per CTA, the kernels' static variables included
+constexpr int kStaticSmem = 64;
+template <int MODE>
+void pair_rings(int nt, int* stages, int* nbuf) {
+  using PC = PairCfg<MODE>;
+  *nbuf = PC::SUB == 1 ? 3 : 2;
+  *stages = 2;
+  while (*stages < PC::MAX_STAGES && PC::smem(nt, *stages + 1, *nbuf) + kStaticSmem <= kMaxSmem) ++*stages;
+}
+
+// Shared-memory opt-in of the tensor-core kernels of a mode, once per device (also called
+// ahead of a graph capture).
+template <int MODE>
 int ensure_tc_attr() {
-  using CF = TcCfg<MODE, SPLITACC>;
   static int attr_done[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && !attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(cgemm_tc_kernel<MODE, SPLITACC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CF::smem(CF::NT_MAX));
+    using FC = FastCfg<MODE>;
+    using PC = PairCfg<MODE>;
+    cudaError_t e = cudaFuncSetAttribute(cgemm_fast_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)FC::smem(FC::NT_MAX));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(cgemm_pair_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kMaxSmem - kStaticSmem);
     if (e != cudaSuccess) return (int)e;
     attr_done[dev] = 1;
   }
   return 0;
 }
 
-template <int MODE, bool SPLITACC>
-int launch_tc_mode(const void* S, int64_t s_stride, const void* B, int64_t b_stride, void* C,
+template <int MODE>
+int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, int64_t b_stride, void* C,
                    int64_t c_stride, int64_t P, int64_t K, int64_t N, int64_t NL, int64_t Sd,
                    int batch, char* scratch, int64_t scratch_stride, int withhold, bool no_tma, int beta,
                    cudaStream_t st) {
   using M_ = Mode<MODE>;
-  using CF = TcCfg<MODE, SPLITACC>;
-  const int Nt = (int)(N < CF::NT_MAX ? N : CF::NT_MAX);   // N % 16 == 0, N <= 256
+  const int64_t nt_max = fast ? FastCfg<MODE>::NT_MAX : PairCfg<MODE>::NT_MAX;
+  const int Nt = (int)(N < nt_max ? N : nt_max);   // N % 16 == 0
   const int KT = (int)(K / M_::KS);
+  if (int err = ensure_tc_attr<MODE>()) return err;
   dim3 sg((unsigned)((N + 127) / 128), KT, batch);
-  split_site_kernel<MODE, SPLITACC><<<sg, 128, 0, st>>>((const float2*)S, s_stride, (int)K, (int)N, Nt,
-                                              scratch, scratch_stride);
+  auto split = fast ? split_site_kernel<MODE, false> : split_site_kernel<MODE, true>;
+  split<<<sg, 128, 0, st>>>((const float2*)S, s_stride, (int)K, (int)N, Nt, scratch, scratch_stride);
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return (int)e;
@@ -701,19 +1127,27 @@ int launch_tc_mode(const void* S, int64_t s_stride, const void* B, int64_t b_str
   a.P = P; a.K = K; a.N = N; a.NL = NL; a.Sd = Sd; a.J = P * Sd;
   a.Nt = Nt;
   a.NHt = (int)(N / Nt);
-  a.JT = (a.J + kRows - 1) / kRows;
+  const int rows = fast ? kRows : 2 * kRows;
+  a.JT = (a.J + rows - 1) / rows;
   a.tiles = (int64_t)batch * a.JT * a.NHt;
   a.withhold_s = withhold;
   a.beta = beta;
-  alignas(64) CUtensorMap tmA;
-  std::memset(&tmA, 0, sizeof(tmA));
-  a.use_tma = 0;
-  if (CF::NBUF > 0 && !no_tma)
-    a.use_tma = make_b_map(&tmA, B, b_stride, batch, P, K, Sd, M_::KS, &a.box_s, &a.box_p) ? 1 : 0;
-  auto kern = cgemm_tc_kernel<MODE, SPLITACC>;
-  if (int err = ensure_tc_attr<MODE, SPLITACC>()) return err;
-  const int64_t grid = a.tiles < num_sms() ? a.tiles : num_sms();
-  kern<<<(unsigned)grid, CF::THREADS, CF::smem(Nt), st>>>(a, tmA);
+  if (fast) {
+    const int64_t grid = a.tiles < num_sms() ? a.tiles : num_sms();
+    cgemm_fast_kernel<MODE><<<(unsigned)grid, FastCfg<MODE>::THREADS, FastCfg<MODE>::smem(Nt), st>>>(a);
+  } else {
+    alignas(64) CUtensorMap tmA;
+    std::memset(&tmA, 0, sizeof(tmA));
+    a.use_tma = !no_tma && make_b_map(&tmA, B, b_stride, batch, P, K, Sd, PairCfg<MODE>::SUB * M_::KS, &a.box_s, &a.box_p) ? 1 : 0;
+    const int64_t pairs = std::min<int64_t>(a.tiles, num_sms() / 2);
+    pair_rings<MODE>(Nt, &a.stages, &a.nbuf);
+    // it starts while split_site_kernel runs, so that the pair's barriers, TMEM and launch
+    // latency are out of the way
+    e = launch_early(cgemm_pair_kernel<MODE>, dim3((unsigned)(2 * pairs)), dim3(PairCfg<MODE>::THREADS),
+                     PairCfg<MODE>::smem(Nt, a.stages, a.nbuf), st, a, tmA);
+    count_launch();
+    return (int)e;
+  }
   count_launch();
   return (int)cudaGetLastError();
 }
@@ -856,20 +1290,14 @@ int launch_step_tc(const void* S, int64_t s_stride, const void* B, int64_t b_str
   const int withhold = (flags & kTcWithhold) ? 1 : 0;
   const bool no_tma = (flags & kTcNoTma) != 0;
   if (precision == QFX_PREC_C3M_BF16X3)
-    return fast ? launch_tc_mode<QFX_PREC_C3M_BF16X3, false>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                             Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st)
-                : launch_tc_mode<QFX_PREC_C3M_BF16X3, true>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                            Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st);
+    return launch_tc_mode<QFX_PREC_C3M_BF16X3>(fast, S, s_stride, B, b_stride, C, c_stride, P, K, N, NL, Sd, batch,
+                                               scratch, scratch_stride, withhold, no_tma, beta, st);
   if (precision == QFX_PREC_C3M_BF16X2)
-    return fast ? launch_tc_mode<QFX_PREC_C3M_BF16X2, false>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                             Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st)
-                : launch_tc_mode<QFX_PREC_C3M_BF16X2, true>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                            Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st);
+    return launch_tc_mode<QFX_PREC_C3M_BF16X2>(fast, S, s_stride, B, b_stride, C, c_stride, P, K, N, NL, Sd, batch,
+                                               scratch, scratch_stride, withhold, no_tma, beta, st);
   if (precision == QFX_PREC_C3M_TF32X3)
-    return fast ? launch_tc_mode<QFX_PREC_C3M_TF32X3, false>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                             Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st)
-                : launch_tc_mode<QFX_PREC_C3M_TF32X3, true>(S, s_stride, B, b_stride, C, c_stride, P, K, N, NL,
-                                                            Sd, batch, scratch, scratch_stride, withhold, no_tma, beta, st);
+    return launch_tc_mode<QFX_PREC_C3M_TF32X3>(fast, S, s_stride, B, b_stride, C, c_stride, P, K, N, NL, Sd, batch,
+                                               scratch, scratch_stride, withhold, no_tma, beta, st);
   return (int)cudaErrorInvalidValue;
 }
 
@@ -884,12 +1312,9 @@ int tc_probe(int precision, int64_t iters, double* tflops, void* stream) {
 int tc_prepare_attributes() {
   (void)tensor_map_encoder();   // resolve the driver entry point outside any capture
   int e = 0;
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X3, true>();
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X3, false>();
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X2, true>();
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X2, false>();
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_TF32X3, true>();
-  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_TF32X3, false>();
+  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X3>();
+  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_BF16X2>();
+  if (!e) e = ensure_tc_attr<QFX_PREC_C3M_TF32X3>();
   return e;
 }
 

@@ -103,6 +103,26 @@ def test_tensor_map_rows_match_register_rows(qfx, prec, shape):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("prec,shape", [("tf32x3", (1, 24, 48, 48, 384)), ("tf32x3", (3, 40, 128, 64, 128)),
+                                        ("tf32x3", (701, 24, 256, 256, 128)), ("bf16x3", (1, 48, 16, 16, 384)),
+                                        ("bf16x3", (5, 16, 80, 40, 128)), ("bf16x2", (257, 32, 112, 112, 128)),
+                                        ("bf16x3", (613, 16, 128, 128, 130)), ("tf32x3", (613, 24, 64, 32, 130))])
+def test_pair_tile_edges(qfx, prec, shape):
+    """The pair tile (256 rows j over two CTAs) at its edges: an odd number of 128-row tiles
+    (the second CTA's last one is empty), an odd number of TF32 k-steps (two to a stage),
+    accumulators that alternate between the halves of the TMEM (N tiles up to 64) or take
+    turns (above), pairs that run several tiles, and rows that no tensor map describes."""
+    P, K, N, NL, Sd = shape
+    S = ri.random_complex((K, N), seed=21)
+    B = ri.random_complex((P, K, Sd), seed=22)
+    want = step_ref(S, B, P, K, N, NL, Sd)
+    dS, dB = torch.from_numpy(S.reshape(-1)).cuda(), torch.from_numpy(B.reshape(-1)).cuda()
+    for v in (-1, 13):
+        got = qfx.contract_step(dS, dB, P, K, N, NL, Sd, precision=prec, variant=v).cpu().numpy().reshape(want.shape)
+        qfx.sync()
+        check_step(got, want, S, B, P, K, N, NL, Sd, STEP_BOUND[prec])
+
+
 @pytest.mark.parametrize("shape", [(1, 8, 64, 64, 4096), (2, 8, 16, 8, 4096), (512, 8, 64, 64, 1),
                                    (40, 8, 32, 32, 4)])
 def test_tf32_single_kstage_steps(qfx, shape):
