@@ -14,6 +14,11 @@ namespace qfx {
 namespace {
 using namespace simt;
 
+__device__ __forceinline__ void simt_cp_async8(float2* smem, const float2* gmem) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem));
+}
+
 template <int BM, int BJ, int TM, int TJ, bool KMODE>
 __global__ void __launch_bounds__(256, 2) cgemm_step_kernel(const StepArgs a) {
   extern __shared__ float4 smem_raw[];
@@ -51,22 +56,77 @@ int launch_cfg(const StepArgs& a, int batch, cudaStream_t stream) {
   return (int)cudaGetLastError();
 }
 
-// Split-K sum of a chunked contraction.  A block covers kRedE consecutive outputs with
-// kRedL lanes each: lane l of an output adds chunks l, l + kRedL, ... in FP64 (a warp reads
-// kRedE-long runs of each chunk's row), then lane 0 adds the lanes' sums in lane order and
-// rounds once to FP32.
-constexpr int kRedE = 32, kRedL = 8;
-__global__ void __launch_bounds__(kRedE * kRedL) reduce_parts_kernel(const float2* __restrict__ part,
-                                                                     int64_t part_stride, int64_t parts,
-                                                                     int64_t out, float2* __restrict__ C,
-                                                                     int64_t c_stride) {
-  __shared__ double2 lanes[kRedL][kRedE];
-  const int el = threadIdx.x % kRedE, lane = threadIdx.x / kRedE;
-  const int64_t e = (int64_t)blockIdx.x * kRedE + el;
+// Chunk products of a split-K contraction with a small result: part c is the N x Sd product
+// (at most kPartsOut outputs) of rows [c * chunk, (c + 1) * chunk) of S and B.  A thread owns one
+// output and walks its chunk's k in order, with the operations of the step tiles, so the
+// result is theirs bit for bit.  The step tiles would fill a row of 512 columns with Sd of them
+// (N = Sd = 8, 2048 chunks of 1024: 1.50 ms; here 0.11); a block takes kPartsOut / (N * Sd)
+// chunks, and slabs of KB rows of both operands arrive by cp.async in two buffers.  The floor is
+// their reading (268 MB, 40 us); the chain of a chunk's k adds to it.
+constexpr int kPartsOut = 256;
+__global__ void __launch_bounds__(kPartsOut) small_parts_kernel(const float2* __restrict__ S,
+                                                               const float2* __restrict__ B,
+                                                               float2* __restrict__ part, int chunk,
+                                                               int64_t parts, int N, int Sd, int KB) {
+  extern __shared__ __align__(16) float2 slab[];
+  const int out = N * Sd, per_block = kPartsOut / out, row = N + Sd;
+  const int own = threadIdx.x / out, e = threadIdx.x - own * out, n = e / Sd, s = e - n * Sd;
+  const int64_t c0 = (int64_t)blockIdx.x * per_block;
+  const int here = (int)min((int64_t)per_block, parts - c0);
+  // buffer: per chunk of the block, KB rows of S, then KB rows of B
+  auto fetch = [&](int k0, int buf) {
+    float2* dst = slab + (int64_t)buf * per_block * KB * row;
+    const int rows = min(KB, chunk - k0);
+    for (int w = 0; w < here; ++w) {
+      const int64_t k = (c0 + w) * chunk + k0;
+      for (int i = threadIdx.x; i < rows * N; i += kPartsOut)
+        simt_cp_async8(dst + (int64_t)w * KB * row + i, S + k * N + i);
+      for (int i = threadIdx.x; i < rows * Sd; i += kPartsOut)
+        simt_cp_async8(dst + (int64_t)w * KB * row + KB * N + i, B + k * Sd + i);
+    }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  float re = 0.f, im = 0.f;
+  fetch(0, 0);
+  for (int k0 = 0, buf = 0; k0 < chunk; k0 += KB, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;\n" ::);
+    __syncthreads();   // this slab landed for every thread; the other buffer is free
+    if (k0 + KB < chunk) fetch(k0 + KB, buf ^ 1);
+    if (own < here) {
+      const float2* Sk = slab + ((int64_t)buf * per_block + own) * KB * row;
+      const float2* Bk = Sk + KB * N;
+      const int rows = min(KB, chunk - k0);
+#pragma unroll 8
+      for (int k = 0; k < rows; ++k) {
+        const float2 a = Sk[k * N + n], b = Bk[k * Sd + s];
+        re = fmaf(a.x, b.x, re);
+        re = fmaf(-a.y, b.y, re);
+        im = fmaf(a.x, b.y, im);
+        im = fmaf(a.y, b.x, im);
+      }
+    }
+  }
+  if (own < here) part[(c0 + own) * out + e] = make_float2(re, im);
+}
+
+// Split-K sum of a chunked contraction.  A block covers E consecutive outputs with kRedL lanes
+// each: lane l of an output adds chunks l, l + kRedL, ... in FP64, then lane 0 adds the lanes'
+// sums in lane order and rounds once to FP32.  FP64 conversions and additions run at two lanes
+// a clock on an SM, so few outputs take blocks of 4 of them, spread over the SMs (64 outputs
+// of 2048 chunks: 42 us, against 78 in blocks of 32); many take 32, whose warps read longer runs.
+constexpr int kRedL = 8;
+template <int E>
+__global__ void __launch_bounds__(E * kRedL) reduce_parts_kernel(const float2* __restrict__ part,
+                                                                 int64_t part_stride, int64_t parts,
+                                                                 int64_t out, float2* __restrict__ C,
+                                                                 int64_t c_stride) {
+  __shared__ double2 lanes[kRedL][E];
+  const int el = threadIdx.x % E, lane = threadIdx.x / E;
+  const int64_t e = (int64_t)blockIdx.x * E + el;
   const float2* pp = part + (int64_t)blockIdx.y * part_stride;
   double re = 0.0, im = 0.0;
   if (e < out) {
-#pragma unroll 4
+#pragma unroll 8
     for (int64_t c = lane; c < parts; c += kRedL) {
       const float2 v = pp[c * out + e];
       re += (double)v.x;
@@ -89,10 +149,31 @@ __global__ void __launch_bounds__(kRedE * kRedL) reduce_parts_kernel(const float
 int launch_reduce_parts(const void* part, int64_t part_stride, int64_t parts, int64_t out, void* C,
                         int64_t c_stride, int batch, void* stream) {
   if (parts < 1 || out < 1 || batch < 1 || batch > 65535) return (int)cudaErrorInvalidValue;
-  const int64_t blocks = (out + kRedE - 1) / kRedE;
+  const bool few = out <= 32 * (int64_t)num_sms();
+  const int64_t blocks = few ? (out + 3) / 4 : (out + 31) / 32;
   if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
-  reduce_parts_kernel<<<dim3((unsigned)blocks, (unsigned)batch), kRedE * kRedL, 0, (cudaStream_t)stream>>>(
+  auto kern = few ? reduce_parts_kernel<4> : reduce_parts_kernel<32>;
+  kern<<<dim3((unsigned)blocks, (unsigned)batch), (few ? 4 : 32) * kRedL, 0, (cudaStream_t)stream>>>(
       (const float2*)part, part_stride, parts, out, (float2*)C, c_stride);
+  count_launch();
+  return (int)cudaGetLastError();
+}
+
+// Whether launch_small_parts takes a split-K contraction of this result.
+bool small_parts_fit(int64_t N, int64_t Sd) { return N * Sd <= kPartsOut; }
+
+int launch_small_parts(const void* S, const void* B, void* part, int64_t chunk, int64_t parts, int64_t N,
+                       int64_t Sd, void* stream) {
+  if (!small_parts_fit(N, Sd) || chunk < 1 || chunk > (1 << 20) || parts < 1) return (int)cudaErrorInvalidValue;
+  const int per_block = kPartsOut / (int)(N * Sd);
+  const int64_t blocks = (parts + per_block - 1) / per_block;
+  if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
+  // rows per slab: two buffers in at most 40 KB (N + Sd <= 257 and per_block = 1 at the widest)
+  const int row = (int)(N + Sd) * per_block * 8;
+  int KB = 64;
+  while (KB > 1 && 2 * KB * row > (40 << 10)) KB /= 2;
+  small_parts_kernel<<<(unsigned)blocks, kPartsOut, (size_t)2 * KB * row, (cudaStream_t)stream>>>(
+      (const float2*)S, (const float2*)B, (float2*)part, (int)chunk, parts, (int)N, (int)Sd, KB);
   count_launch();
   return (int)cudaGetLastError();
 }

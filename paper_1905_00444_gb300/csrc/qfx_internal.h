@@ -209,6 +209,9 @@ bool simt_variant_valid(int variant, int64_t Sd);
 int num_sms();
 // C[b][e] = sum over c < parts of part[b][c][e] (e < out; complex FP32 in and out), per batch
 // entry b < batch, in FP64 and a fixed order; strides in float2 units.
+bool small_parts_fit(int64_t N, int64_t Sd);
+int launch_small_parts(const void* S, const void* B, void* part, int64_t chunk, int64_t parts, int64_t N,
+                       int64_t Sd, void* stream);
 int launch_reduce_parts(const void* part, int64_t part_stride, int64_t parts, int64_t out, void* C,
                         int64_t c_stride, int batch, void* stream);
 // tensor-core steps (variants 10 = BF16x3, 11 = TF32x3)

@@ -254,9 +254,13 @@ static qfx_status exec_tree(const qfx_plan* p, const DeviceTables& t, const uint
         // split K: chunk c's product into part[c] (the item's scratch), then the sum into C
         for (int gi = 0; gi < g && !err; ++gi) {
           char* blk = items + (uint64_t)gi * ib;
-          err = launch_step(blk + nd.offA2, nd.chunk * nd.N, blk + nd.offB2, nd.chunk * nd.Sd,
-                            blk + L.simage, nd.N * nd.Sd, 1, nd.chunk, nd.N, nd.NL, nd.Sd, nd.parts,
-                            fill_variant(nd.variant, nd.N, nd.Sd, nd.parts), QFX_PREC_FP32_SIMT, st, 0);
+          if (small_parts_fit(nd.N, nd.Sd))
+            err = launch_small_parts(blk + nd.offA2, blk + nd.offB2, blk + L.simage, nd.chunk, nd.parts, nd.N,
+                                     nd.Sd, st);
+          else
+            err = launch_step(blk + nd.offA2, nd.chunk * nd.N, blk + nd.offB2, nd.chunk * nd.Sd,
+                              blk + L.simage, nd.N * nd.Sd, 1, nd.chunk, nd.N, nd.NL, nd.Sd, nd.parts,
+                              fill_variant(nd.variant, nd.N, nd.Sd, nd.parts), QFX_PREC_FP32_SIMT, st, 0);
         }
         if (!err)
           err = launch_reduce_parts(items + L.simage, (int64_t)(ib / 8), nd.parts, nd.N * nd.Sd,

@@ -109,6 +109,20 @@ def test_split_k_nodes_vs_oracle(qfx, shape):
     check(out, want, rows * cols)
 
 
+@pytest.mark.parametrize("depth,n_open", [(32, 1), (32, 3), (32, 7), (32, 8), (32, 9), (40, 0), (40, 5)])
+def test_small_split_k_results(qfx, depth, n_open):
+    # roots of 1 to 512 outputs: one thread per output up to 256 of them, parts that fill a
+    # block unevenly (4 parts, 256 a block), the step tiles above; every amplitude against the
+    # state vector at the FP32 bar
+    c = ri.rqc(4, 4, depth, seed=2)
+    plan = qfx.Plan(qfx.Circuit(c), n_open=n_open, family="tree")
+    assert any(s["parts"] > 0 and s["N"] * s["Sd"] == 1 << n_open for s in plan.steps)
+    x1s = ri.random_bitstrings(16, 2, seed=9)
+    psi = statevector.amplitudes(c)
+    want = np.array([[psi[expand(x, plan.open_sites, j)] for j in range(1 << n_open)] for x in x1s])
+    check(run(qfx, plan, x1s, items=2), want, 16)
+
+
 def test_general_two_qubit_gates(qfx):
     c = ri.rqc(4, 4, 8, seed=3, two_qubit="fsim")
     plan = qfx.Plan(qfx.Circuit(c), n_open=4, family="tree")
