@@ -26,6 +26,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fold_element.cuh"
 #include "qfx_internal.h"
 
 namespace qfx {
@@ -425,11 +426,8 @@ __global__ void __launch_bounds__(kT) fold_backward_kernel(
       if (st.edge[s] == cd.edge) off[s] = digit * cd.size;
   }
   int64_t r = active ? i : 0;
-  const int64_t vd = r % st.dim[4]; r /= st.dim[4];
-  const int64_t vr = r % st.dim[3]; r /= st.dim[3];
-  const int64_t vx = r % st.dim[2]; r /= st.dim[2];
-  const int64_t vl = r % st.dim[1]; r /= st.dim[1];
-  const int64_t vu = r;
+  const int64_t vd = foldk::take_bits(r, st.dim[4]), vr = foldk::take_bits(r, st.dim[3]);
+  const int64_t vx = foldk::take_bits(r, st.dim[2]), vl = foldk::take_bits(r, st.dim[1]), vu = r;
   const uint64_t val0 = (uint64_t)(vu + off[0]), val1 = (uint64_t)(vl + off[1]);
   const uint64_t val2 = (uint64_t)(vr + off[2]), val3 = (uint64_t)(vd + off[3]);
   const int xv = st.x_open ? (int)vx : (int)((x1w[st.qubit >> 6] >> (st.qubit & 63)) & 1ull);

@@ -178,12 +178,36 @@ __global__ void __launch_bounds__(kT, 2) batch_kernel(const BatchArgs a) {
       const int64_t end = min(st.size, start + kFoldChunk);
       float2* T = sites + st.offset;
       if (sg.phase == PH_FOLD) {
+        // an element per thread and pass (the results are those of fold_kernel, which do not
+        // depend on how elements are grouped); the events are staged once when they fit
         float mx = 0.f;
-        for (int64_t i = start + tid; i < end; i += kT) {
-          const float2 v = foldk::fold_element(st, pl.t.events, pl.t.matsf, pl.t.cuts, pl.n_cuts,
-                                               w.x1, w.sid, i);
-          T[i] = v;
-          mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+        foldk::FoldStage& sm = *reinterpret_cast<foldk::FoldStage*>(smem);
+        const int nev = st.ev_end - st.ev_begin;
+        const bool once = nev <= foldk::kFoldStage;
+        if (once) {
+          foldk::stage_events(sm, pl.t.events, pl.t.matsf, st.ev_begin, nev, tid, kT);
+          __syncthreads();
+        }
+        for (int64_t i0 = start; i0 < end; i0 += kT) {   // block-uniform
+          const int64_t i = i0 + tid;
+          foldk::FoldState<1> f;
+          f.begin(st, pl.t.cuts, pl.n_cuts, w.x1, w.sid, i < end ? i : 0);
+          if (once) {
+            f.run(sm, pl.t.matsf, nev);
+          } else {
+            for (int e0 = st.ev_begin; e0 < st.ev_end; e0 += foldk::kFoldStage) {
+              const int n = min(foldk::kFoldStage, st.ev_end - e0);
+              __syncthreads();
+              foldk::stage_events(sm, pl.t.events, pl.t.matsf, e0, n, tid, kT);
+              __syncthreads();
+              f.run(sm, pl.t.matsf, n);
+            }
+          }
+          if (i < end) {
+            const float2 v = f.result(0);
+            T[i] = v;
+            mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+          }
         }
         const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
         if ((tid & 31) == 0) s_max[tid >> 5] = __uint_as_float(bits);

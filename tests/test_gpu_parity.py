@@ -233,6 +233,20 @@ def test_7x7x32_one_full_bond_cut_16_slices(qfx):
     assert np.all(np.abs(sliced - full) <= REL * np.maximum(np.abs(full), floor))
 
 
+@pytest.mark.parametrize("shape,kind", [((4, 4, 16), "cz"), ((2, 3, 56), "cz"), ((3, 3, 8), "fsim")])
+def test_fold_of_one_item_and_of_many(qfx, shape, kind):
+    """One item folds an element per thread, many items groups of 4 (sites of one element and
+    of thousands among them); (2, 3, 56) has more events per site than one stage in shared
+    memory holds.  The grouping never changes a bit, and so neither do the amplitudes."""
+    rows, cols, d = shape
+    plan = qfx.Plan(qfx.Circuit(ri.rqc(rows, cols, d, seed=5, two_qubit=kind)), n_open=2)
+    x1 = torch.tensor(ri.random_bitstrings(rows * cols, 160, seed=6).view(np.int64), device="cuda")
+    many = qfx.amplitudes(plan, x1, workspace=torch.empty(plan.workspace_bytes(160), dtype=torch.uint8, device="cuda"))
+    one = torch.cat([qfx.amplitudes(plan, x1[i:i + 1]) for i in range(0, 160, 53)])
+    qfx.sync()
+    assert torch.equal(many[::53], one)
+
+
 # --- single operations: contraction step and permute --------------------------------
 
 FILL = {0: 20, 1: 20, 2: 21, 3: 22, 4: 23, 5: 25, 6: 25, 7: 26, 8: 27, 9: 28}
