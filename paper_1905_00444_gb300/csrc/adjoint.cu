@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "fold_element.cuh"
+#include "launch.cuh"
 #include "qfx_internal.h"
 
 namespace qfx {
@@ -40,8 +41,10 @@ uint64_t a256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
 
 // ---- seed: R_n[f(o)] = gbar[o] * 2^-m ------------------------------------------------
-__global__ void __launch_bounds__(kT) seed_kernel(const double* __restrict__ gout, const int32_t* __restrict__ open_perm,
+__global__ void __launch_bounds__(kT) seed_kernel(const double* gout, const int32_t* __restrict__ open_perm,
                                                   int n_open, float2* R, int* m_out) {
+  launch_next();
+  launch_wait();
   __shared__ double red[kT];
   const int64_t per = int64_t(1) << n_open;
   double mx = 0.0;
@@ -65,9 +68,10 @@ __global__ void __launch_bounds__(kT) seed_kernel(const double* __restrict__ gou
 // ---- reverse step: Rout[p][k][s] = sum_n conj(S[k][n]) Rin[n/NL][p][n%NL][s] ------------
 // BM (16 or 64) rows k by 64 columns j per block; thread (ty, tx) owns BM/16 x 4 outputs.
 template <int BM>
-__global__ void __launch_bounds__(kT) rstep_kernel(const float2* __restrict__ S, const float2* __restrict__ Rin,
-                                                   float2* __restrict__ Rout, int64_t P, int64_t K,
+__global__ void __launch_bounds__(kT) rstep_kernel(const float2* S, const float2* Rin, float2* Rout, int64_t P, int64_t K,
                                                    int64_t N, int64_t NL, int64_t Sd) {
+  launch_next();
+  launch_wait();
   constexpr int BJ = 64, BR = 16, TMK = BM / 16;
   static_assert(kT == 256 && (BM == 16 || BM == 64), "thread layout");
   __shared__ float2 As[BR][BM + 1];
@@ -152,8 +156,9 @@ struct ConjTable {
   int32_t K[kConjMax], N[kConjMax];
   int32_t count;
 };
-__global__ void __launch_bounds__(kT) conj_transpose_kernel(const float2* __restrict__ sites,
-                                                            float2* __restrict__ sconj, const ConjTable tab) {
+__global__ void __launch_bounds__(kT) conj_transpose_kernel(const float2* sites, float2* sconj, const ConjTable tab) {
+  launch_next();
+  launch_wait();
   __shared__ float2 tile[32][33];
   const int y = blockIdx.y;
   const int64_t K = tab.K[y], N = tab.N[y];
@@ -182,12 +187,11 @@ int launch_rstep(const float2* S, const float2* Rin, float2* Rout, int64_t P, in
   const int64_t J = P * Sd;
   if (K <= 16) {
     const int64_t blocks = ((K + 15) / 16) * ((J + 63) / 64);
-    rstep_kernel<16><<<(unsigned)blocks, kT, 0, st>>>(S, Rin, Rout, P, K, N, NL, Sd);
+    return (int)launch_early(rstep_kernel<16>, dim3((unsigned)blocks), dim3(kT), 0, st, S, Rin, Rout, P, K, N, NL, Sd);
   } else {
     const int64_t blocks = ((K + 63) / 64) * ((J + 63) / 64);
-    rstep_kernel<64><<<(unsigned)blocks, kT, 0, st>>>(S, Rin, Rout, P, K, N, NL, Sd);
+    return (int)launch_early(rstep_kernel<64>, dim3((unsigned)blocks), dim3(kT), 0, st, S, Rin, Rout, P, K, N, NL, Sd);
   }
-  return (int)cudaGetLastError();
 }
 
 // ---- site gradient, split over columns: part[c][k][n] = sum_{j in c} conj(L(k,j)) R(n,j) ----
@@ -202,9 +206,10 @@ __device__ __forceinline__ void g_cp_async8(void* smem, const void* gmem, bool p
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(pred ? 8 : 0));
 }
 template <int BM, int BN>
-__global__ void __launch_bounds__(kT) grads_kernel(const float2* __restrict__ Lin, const float2* __restrict__ Rin,
-                                                   float2* __restrict__ part, int64_t P, int64_t K,
+__global__ void __launch_bounds__(kT) grads_kernel(const float2* Lin, const float2* Rin, float2* part, int64_t P, int64_t K,
                                                    int64_t N, int64_t NL, int64_t Sd, int64_t chunk) {
+  launch_next();
+  launch_wait();
   constexpr int BJ = 16, TMK = BM / 16, TNN = BN / 16;
   constexpr int LA = BM + 2, LB = BN + 2;   // rows of 16-byte multiples, 2-way store conflicts
   static_assert(kT == 256 && BM % 16 == 0 && BN % 16 == 0, "thread layout");
@@ -327,17 +332,17 @@ GradsGeom grads_geom(int64_t K, int64_t N, int64_t J) {
 int launch_grads(const GradsGeom& g, const float2* Lin, const float2* Rin, float2* part, int64_t P, int64_t K,
                  int64_t N, int64_t NL, int64_t Sd, cudaStream_t st) {
   dim3 grid((unsigned)((K + g.bm - 1) / g.bm), (unsigned)((N + g.bn - 1) / g.bn), (unsigned)g.chunks);
-  if (g.bm == 16 && g.bn == 16) grads_kernel<16, 16><<<grid, kT, 0, st>>>(Lin, Rin, part, P, K, N, NL, Sd, g.chunk);
-  else if (g.bm == 16) grads_kernel<16, 64><<<grid, kT, 0, st>>>(Lin, Rin, part, P, K, N, NL, Sd, g.chunk);
-  else if (g.bn == 16) grads_kernel<64, 16><<<grid, kT, 0, st>>>(Lin, Rin, part, P, K, N, NL, Sd, g.chunk);
-  else grads_kernel<64, 64><<<grid, kT, 0, st>>>(Lin, Rin, part, P, K, N, NL, Sd, g.chunk);
-  return (int)cudaGetLastError();
+  auto kern = g.bm == 16 ? (g.bn == 16 ? grads_kernel<16, 16> : grads_kernel<16, 64>)
+                         : (g.bn == 16 ? grads_kernel<64, 16> : grads_kernel<64, 64>);
+  return (int)launch_early(kern, grid, dim3(kT), 0, st, Lin, Rin, part, P, K, N, NL, Sd, g.chunk);
 }
 
 // One warp per output element: lane l sums chunks l, l + 32, ... in order, then a fixed
 // butterfly adds the lanes (deterministic).
-__global__ void __launch_bounds__(kT) reduce_chunks_kernel(const float2* __restrict__ part, int64_t chunks,
-                                                           int64_t KN, float2* __restrict__ out) {
+__global__ void __launch_bounds__(kT) reduce_chunks_kernel(const float2* part, int64_t chunks,
+                                                           int64_t KN, float2* out) {
+  launch_next();
+  launch_wait();
   const int64_t t = ((int64_t)blockIdx.x * kT + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= KN) return;   // warp-uniform: t is the same for all lanes of a warp
@@ -409,7 +414,9 @@ __host__ __device__ __forceinline__ int ev_slots(int kind) { return kind == EV_B
 __global__ void __launch_bounds__(kT) fold_backward_kernel(
     const FoldSite* __restrict__ sites, const FoldEvent* __restrict__ events, const float* __restrict__ matsf,
     const CutDev* __restrict__ cuts, int n_cuts, const uint64_t* __restrict__ x1w, int64_t sid,
-    const float2* __restrict__ sgrad, double* __restrict__ bpart, const int64_t* __restrict__ part_off) {
+    const float2* sgrad, double* bpart, const int64_t* __restrict__ part_off) {
+  launch_next();
+  launch_wait();
   __shared__ double wpart[kT / 32][kMaxEvents][8];
   const FoldSite st = sites[blockIdx.y];
   const int nev = st.ev_end - st.ev_begin;
@@ -536,10 +543,12 @@ __global__ void __launch_bounds__(kT) fold_backward_kernel(
 // 2^(E - e_s + m); evgrad holds 32 doubles per event
 __global__ void __launch_bounds__(kT) event_reduce_kernel(const FoldSite* __restrict__ sites, int n_sites,
                                                           const FoldEvent* __restrict__ events,
-                                                          const double* __restrict__ bpart,
+                                                          const double* bpart,
                                                           const int64_t* __restrict__ part_off,
-                                                          const int* __restrict__ hdr_exps, const int* m_ptr,
-                                                          int n_events, double* __restrict__ evgrad) {
+                                                          const int* hdr_exps, const int* m_ptr,
+                                                          int n_events, double* evgrad) {
+  launch_next();
+  launch_wait();
   const int t = blockIdx.x * kT + threadIdx.x;
   if (t >= n_events * 32) return;
   const int e = t / 32, entry = t % 32;
@@ -570,8 +579,10 @@ __global__ void __launch_bounds__(kT) event_reduce_kernel(const FoldSite* __rest
 // fill their first 4 entries.
 __global__ void __launch_bounds__(kT) gate_accum_kernel(const int32_t* __restrict__ gate_ev,
                                                         const FoldEvent* __restrict__ events, int n_gates,
-                                                        int per_gate, const double* __restrict__ evgrad,
+                                                        int per_gate, const double* evgrad,
                                                         double* grad) {
+  launch_next();
+  launch_wait();
   const int t = blockIdx.x * kT + threadIdx.x;
   if (t >= n_gates * 2 * per_gate) return;
   const int gte = t / (2 * per_gate), ent = t % (2 * per_gate), ce = ent / 2, ri = ent & 1;
@@ -742,9 +753,10 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
     if (!err) err = launch_scale(t, n, max_site, 1, hdr, 0, sites, 0, 0, st);
     if (err) return cuda_fail(err, "qfx_amplitudes_backward: fold");
     if (ctab.count > 0) {
-      conj_transpose_kernel<<<dim3((unsigned)conj_tiles, (unsigned)ctab.count), kT, 0, st>>>(
-          (const float2*)sites, sconj, ctab);
+      err = (int)launch_early(conj_transpose_kernel, dim3((unsigned)conj_tiles, (unsigned)ctab.count), dim3(kT), 0, st,
+                              (const float2*)sites, sconj, ctab);
       count_launch();
+      if (err) return cuda_fail(err, "qfx_amplitudes_backward: conjugate transposes");
     }
     // forward sweep, keeping every step's output (full) or the boundary at the start of
     // every line
@@ -760,8 +772,9 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
     // seed from this batch row's upstream gradient
     float2* Rcur = (float2*)rr(0);
     int rsel = 0;
-    seed_kernel<<<1, kT, 0, st>>>(grad_out + 2 * b * per, t.open_perm, n_open, Rcur, m_ptr);
+    err = (int)launch_early(seed_kernel, dim3(1), dim3(kT), 0, st, grad_out + 2 * b * per, t.open_perm, n_open, Rcur, m_ptr);
     count_launch();
+    if (err) return cuda_fail(err, "qfx_amplitudes_backward: seed");
     // reverse: gradient of step i's site from its input Lin and the incoming R, then R
     // through the step
     auto reverse_step = [&](int i, const char* Lin_raw) -> qfx_status {
@@ -776,18 +789,22 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
       const int64_t J = sp.P * sp.Sd;
       const GradsGeom gg = grads_geom(sp.K, sp.N, J);
       float2* part = (float2*)(ws + Lw.gpart);
-      launch_grads(gg, Lin, Rcur, part, sp.P, sp.K, sp.N, sp.NL, sp.Sd, st);
+      int err2 = launch_grads(gg, Lin, Rcur, part, sp.P, sp.K, sp.N, sp.NL, sp.Sd, st);
       const int64_t KN = sp.K * sp.N;
-      reduce_chunks_kernel<<<(unsigned)((KN * 32 + kT - 1) / kT), kT, 0, st>>>(part, gg.chunks, KN, gdst);
+      if (!err2)
+        err2 = (int)launch_early(reduce_chunks_kernel, dim3((unsigned)((KN * 32 + kT - 1) / kT)), dim3(kT), 0, st,
+                                 part, gg.chunks, KN, gdst);
+      if (err2) return cuda_fail(err2, "qfx_amplitudes_backward: site gradient");
       float2* Rnext = (float2*)rr(rsel ^ 1);
       if (use_conj[i]) {
         const int v = fill_variant(pick_variant(sp.K, sp.Sd), sp.K, J, 1);
-        const int err2 = launch_step(sconj + p->sites[sp.site].offset, 0, Rcur, 0, Rnext, 0, sp.P, sp.N, sp.K,
+        err2 = launch_step(sconj + p->sites[sp.site].offset, 0, Rcur, 0, Rnext, 0, sp.P, sp.N, sp.K,
                                      sp.K, sp.Sd, 1, v, QFX_PREC_FP32_SIMT, st);
         if (err2) return cuda_fail(err2, "qfx_amplitudes_backward: reverse step");
         count_launch(2);
       } else {
-        launch_rstep((const float2*)site_ptr(sp.site), Rcur, Rnext, sp.P, sp.K, sp.N, sp.NL, sp.Sd, st);
+        err2 = launch_rstep((const float2*)site_ptr(sp.site), Rcur, Rnext, sp.P, sp.K, sp.N, sp.NL, sp.Sd, st);
+        if (err2) return cuda_fail(err2, "qfx_amplitudes_backward: reverse step");
         count_launch(3);
       }
       rsel ^= 1;
@@ -826,18 +843,17 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
     }
     // back through every site's time fold
     dim3 fg((unsigned)((max_site + kT - 1) / kT), n);
-    fold_backward_kernel<<<fg, kT, 0, st>>>(t.sites, t.events, t.matsf, t.cuts, (int)p->cut_dev.size(),
-                                            x1 + b * p->x1_words, sid, sgrad, (double*)(ws + Lw.bpart),
-                                            t.partoff);
+    e = launch_early(fold_backward_kernel, fg, dim3(kT), 0, st, t.sites, t.events, t.matsf, t.cuts,
+                     (int)p->cut_dev.size(), x1 + b * p->x1_words, sid, sgrad, (double*)(ws + Lw.bpart), t.partoff);
     const int nev = (int)p->events.size();
-    event_reduce_kernel<<<(nev * 32 + kT - 1) / kT, kT, 0, st>>>(t.sites, n, t.events,
-                                                                (const double*)(ws + Lw.bpart),
-                                                                t.partoff, exps,
-                                                                m_ptr, nev, (double*)(ws + Lw.evgrad));
-    gate_accum_kernel<<<(p->n_gates * 2 * per_gate + kT - 1) / kT, kT, 0, st>>>(
-        t.gate_ev, t.events, p->n_gates, per_gate, (const double*)(ws + Lw.evgrad), grad_gates);
+    if (e == cudaSuccess)
+      e = launch_early(event_reduce_kernel, dim3((nev * 32 + kT - 1) / kT), dim3(kT), 0, st, t.sites, n, t.events,
+                       (const double*)(ws + Lw.bpart), t.partoff, exps, m_ptr, nev, (double*)(ws + Lw.evgrad));
+    if (e == cudaSuccess)
+      e = launch_early(gate_accum_kernel, dim3((p->n_gates * 2 * per_gate + kT - 1) / kT), dim3(kT), 0, st, t.gate_ev,
+                       t.events, p->n_gates, per_gate, (const double*)(ws + Lw.evgrad), grad_gates);
     count_launch(3);
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes_backward: fold adjoint");
   }
   return QFX_OK;

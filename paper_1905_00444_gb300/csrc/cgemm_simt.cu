@@ -8,6 +8,7 @@
 #include <cstdio>
 
 #include "cgemm_tile.cuh"
+#include "launch.cuh"
 #include "qfx_internal.h"
 
 namespace qfx {
@@ -21,6 +22,8 @@ __device__ __forceinline__ void simt_cp_async8(float2* smem, const float2* gmem)
 
 template <int BM, int BJ, int TM, int TJ, bool KMODE>
 __global__ void __launch_bounds__(256, 2) cgemm_step_kernel(const StepArgs a) {
+  launch_next();
+  launch_wait();
   extern __shared__ float4 smem_raw[];
   cgemm_tile<BM, BJ, TM, TJ, KMODE>(a, blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -51,9 +54,8 @@ int launch_cfg(const StepArgs& a, int batch, cudaStream_t stream) {
   const int64_t JT = (a.J + BJ - 1) / BJ;
   const int64_t blocks = NT * JT;
   if (blocks > 0x7fffffffLL || batch > 65535) return (int)cudaErrorInvalidConfiguration;
-  kern<<<dim3((unsigned)blocks, batch), 256, C_::SMEM, stream>>>(a);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(kern, dim3((unsigned)blocks, batch), dim3(256), C_::SMEM, stream, a);
 }
 
 // Chunk products of a split-K contraction with a small result: part c is the N x Sd product
@@ -64,10 +66,10 @@ int launch_cfg(const StepArgs& a, int batch, cudaStream_t stream) {
 // chunks, and slabs of KB rows of both operands arrive by cp.async in two buffers.  The floor is
 // their reading (268 MB, 40 us); the chain of a chunk's k adds to it.
 constexpr int kPartsOut = 256;
-__global__ void __launch_bounds__(kPartsOut) small_parts_kernel(const float2* __restrict__ S,
-                                                               const float2* __restrict__ B,
-                                                               float2* __restrict__ part, int chunk,
+__global__ void __launch_bounds__(kPartsOut) small_parts_kernel(const float2* S, const float2* B, float2* part, int chunk,
                                                                int64_t parts, int N, int Sd, int KB) {
+  launch_next();
+  launch_wait();
   extern __shared__ __align__(16) float2 slab[];
   const int out = N * Sd, per_block = kPartsOut / out, row = N + Sd;
   const int own = threadIdx.x / out, e = threadIdx.x - own * out, n = e / Sd, s = e - n * Sd;
@@ -116,10 +118,11 @@ __global__ void __launch_bounds__(kPartsOut) small_parts_kernel(const float2* __
 // of 2048 chunks: 42 us, against 78 in blocks of 32); many take 32, whose warps read longer runs.
 constexpr int kRedL = 8;
 template <int E>
-__global__ void __launch_bounds__(E * kRedL) reduce_parts_kernel(const float2* __restrict__ part,
+__global__ void __launch_bounds__(E * kRedL) reduce_parts_kernel(const float2* part,
                                                                  int64_t part_stride, int64_t parts,
-                                                                 int64_t out, float2* __restrict__ C,
-                                                                 int64_t c_stride) {
+                                                                 int64_t out, float2* C, int64_t c_stride) {
+  launch_next();
+  launch_wait();
   __shared__ double2 lanes[kRedL][E];
   const int el = threadIdx.x % E, lane = threadIdx.x / E;
   const int64_t e = (int64_t)blockIdx.x * E + el;
@@ -153,10 +156,9 @@ int launch_reduce_parts(const void* part, int64_t part_stride, int64_t parts, in
   const int64_t blocks = few ? (out + 3) / 4 : (out + 31) / 32;
   if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
   auto kern = few ? reduce_parts_kernel<4> : reduce_parts_kernel<32>;
-  kern<<<dim3((unsigned)blocks, (unsigned)batch), (few ? 4 : 32) * kRedL, 0, (cudaStream_t)stream>>>(
-      (const float2*)part, part_stride, parts, out, (float2*)C, c_stride);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(kern, dim3((unsigned)blocks, (unsigned)batch), dim3((few ? 4 : 32) * kRedL), 0,
+                           (cudaStream_t)stream, (const float2*)part, part_stride, parts, out, (float2*)C, c_stride);
 }
 
 // Whether launch_small_parts takes a split-K contraction of this result.
@@ -172,10 +174,10 @@ int launch_small_parts(const void* S, const void* B, void* part, int64_t chunk, 
   const int row = (int)(N + Sd) * per_block * 8;
   int KB = 64;
   while (KB > 1 && 2 * KB * row > (40 << 10)) KB /= 2;
-  small_parts_kernel<<<(unsigned)blocks, kPartsOut, (size_t)2 * KB * row, (cudaStream_t)stream>>>(
-      (const float2*)S, (const float2*)B, (float2*)part, (int)chunk, parts, (int)N, (int)Sd, KB);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(small_parts_kernel, dim3((unsigned)blocks), dim3(kPartsOut), (size_t)2 * KB * row,
+                           (cudaStream_t)stream, (const float2*)S, (const float2*)B, (float2*)part, (int)chunk,
+                           parts, (int)N, (int)Sd, KB);
 }
 
 int simt_prepare_attributes() {

@@ -702,6 +702,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   cluster_barrier();   // barriers of both CTAs initialised, TMEM allocated in both
+  launch_next();
   launch_wait();       // the site image is written
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_slot;
@@ -1009,12 +1010,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
 //     and [Si_t; -Sr_t] are contiguous 2 Nt-row operands (complex product embedded in N);
 //   otherwise: Sr terms then Si terms.
 template <int MODE, bool EMB>
-__global__ void __launch_bounds__(128) split_site_kernel(const float2* __restrict__ S, int64_t s_stride,
+__global__ void __launch_bounds__(128) split_site_kernel(const float2* S, int64_t s_stride,
                                                           int K, int N, int Nt, char* image,
                                                           int64_t img_stride) {
   using M_ = Mode<MODE>;
   constexpr int TERMS = M_::TERMS, KS = M_::KS;
   launch_next();
+  launch_wait();
   const int n = blockIdx.x * 128 + threadIdx.x;
   const int ks = blockIdx.y;
   const int g = blockIdx.z;
@@ -1116,9 +1118,9 @@ int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, in
   if (int err = ensure_tc_attr<MODE>()) return err;
   dim3 sg((unsigned)((N + 127) / 128), KT, batch);
   auto split = fast ? split_site_kernel<MODE, false> : split_site_kernel<MODE, true>;
-  split<<<sg, 128, 0, st>>>((const float2*)S, s_stride, (int)K, (int)N, Nt, scratch, scratch_stride);
+  cudaError_t e = launch_early(split, sg, dim3(128), 0, st, (const float2*)S, s_stride, (int)K, (int)N, Nt, scratch,
+                               scratch_stride);
   count_launch();
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return (int)e;
   TcArgs a{};
   a.B = (const float2*)B; a.b_stride = b_stride;

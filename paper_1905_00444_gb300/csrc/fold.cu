@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "fold_element.cuh"
+#include "launch.cuh"
 #include "qfx_internal.h"
 
 namespace qfx {
@@ -35,6 +36,8 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(
     const uint64_t* __restrict__ x1, int x1_words, int64_t n_batch, int64_t slice_begin,
     int64_t item0, char* hdr, uint64_t hdr_stride, char* items, uint64_t item_bytes,
     uint64_t sites_off, int n_sites) {
+  launch_next();
+  launch_wait();
   __shared__ foldk::FoldStage sm;
   const FoldSite st = sites[blockIdx.y];
   const int g = blockIdx.z;
@@ -73,6 +76,8 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(
 __global__ void __launch_bounds__(kThreads) scale_kernel(
     const FoldSite* __restrict__ sites, char* hdr, uint64_t hdr_stride, char* items,
     uint64_t item_bytes, uint64_t sites_off, int n_sites) {
+  launch_next();
+  launch_wait();
   const FoldSite st = sites[blockIdx.y];
   const int g = blockIdx.z;
   const unsigned* maxabs = reinterpret_cast<const unsigned*>(hdr + (uint64_t)g * hdr_stride);
@@ -97,6 +102,8 @@ __global__ void __launch_bounds__(kThreads) accumulate_kernel(
     const int32_t* __restrict__ open_perm, int n_open, int n_sites, int64_t n_batch,
     int64_t item0, int items, const char* hdr, uint64_t hdr_stride, const char* itemsp,
     uint64_t item_bytes, uint64_t final_off, double* out) {
+  launch_next();
+  launch_wait();
   const int64_t per = int64_t(1) << n_open;
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= n_batch * per) return;
@@ -135,21 +142,19 @@ int launch_fold(const DeviceTables& t, int n_sites, int64_t max_site_size, int n
   const int64_t per_block = (int64_t)kThreads * G;
   dim3 grid((unsigned)((max_site_size + per_block - 1) / per_block), n_sites, items);
   auto kern = G == 4 ? fold_kernel<4> : fold_kernel<1>;
-  kern<<<grid, kThreads, 0, (cudaStream_t)stream>>>(
-      t.sites, t.events, t.matsf, t.cuts, n_cuts, x1, x1_words, n_batch, slice_begin, item0, hdr,
-      hdr_stride, itemsp, item_bytes, sites_off, n_sites);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(kern, grid, dim3(kThreads), 0, (cudaStream_t)stream, t.sites, t.events, t.matsf, t.cuts,
+                           n_cuts, x1, x1_words, n_batch, slice_begin, item0, hdr, hdr_stride, itemsp, item_bytes,
+                           sites_off, n_sites);
 }
 
 int launch_scale(const DeviceTables& t, int n_sites, int64_t max_site_size, int items,
                  char* hdr, uint64_t hdr_stride, char* itemsp, uint64_t item_bytes,
                  uint64_t sites_off, void* stream) {
   dim3 grid((unsigned)((max_site_size + kThreads - 1) / kThreads), n_sites, items);
-  scale_kernel<<<grid, kThreads, 0, (cudaStream_t)stream>>>(t.sites, hdr, hdr_stride, itemsp,
-                                                             item_bytes, sites_off, n_sites);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(scale_kernel, grid, dim3(kThreads), 0, (cudaStream_t)stream, t.sites, hdr, hdr_stride,
+                           itemsp, item_bytes, sites_off, n_sites);
 }
 
 int launch_accumulate(const DeviceTables& t, int n_sites, int n_open, int64_t n_batch,
@@ -158,11 +163,10 @@ int launch_accumulate(const DeviceTables& t, int n_sites, int n_open, int64_t n_
                       void* stream) {
   const int64_t total = n_batch << n_open;
   const unsigned blocks = (unsigned)((total + kThreads - 1) / kThreads);
-  accumulate_kernel<<<blocks, kThreads, 0, (cudaStream_t)stream>>>(
-      t.open_perm, n_open, n_sites, n_batch, item0, items, hdr, hdr_stride, itemsp, item_bytes,
-      final_off, out);
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)launch_early(accumulate_kernel, dim3(blocks), dim3(kThreads), 0, (cudaStream_t)stream, t.open_perm,
+                           n_open, n_sites, n_batch, item0, items, hdr, hdr_stride, itemsp, item_bytes, final_off,
+                           out);
 }
 
 }  // namespace qfx

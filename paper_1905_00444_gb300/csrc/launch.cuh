@@ -3,6 +3,8 @@
 // touches any global memory, until the kernels ahead of it have completed and their writes
 // are visible; a kernel that lets its successor start early says so once its own blocks are
 // running.  Between the small kernels of a sweep this hides most of the launch latency.
+// Such a kernel declares inputs that an earlier one writes without __restrict__: loads that the
+// compiler takes for invariant may move above the wait.
 #pragma once
 
 #include <cuda_runtime.h>
