@@ -9,24 +9,43 @@ from typing import Optional, Sequence
 from . import qfx
 
 
+class _Rebuilt:
+    """A template circuit with its gate matrices replaced by the rows of `mats` ([n, 4] or
+    [n, 16]): 2x2 for a single-qubit gate, 4 diagonal entries for a diagonal two-qubit gate
+    (its first 4 values), 4x4 for a general one (16 values)."""
+
+    def __init__(self, template, mats):
+        self.rows, self.cols, self._template_gates, self._mats = template.rows, template.cols, template.gates, mats
+
+    @property
+    def gates(self):
+        """The gates as objects of the template's kind, with their own matrices."""
+        out = []
+        for g, m in zip(self._template_gates, self._mats):
+            g2 = copy.copy(g)
+            if g.q1 < 0:
+                g2.mat = m[:4].reshape(2, 2).copy()
+            elif g.mat.size == 16:
+                g2.mat = m.reshape(4, 4).copy()
+            else:
+                g2.mat = m[:4].reshape(4).copy()
+            out.append(g2)
+        return out
+
+    def compile(self):
+        """The library's circuit, straight from the rows (an object per gate and step took most
+        of a training step's time on 6x6x(1+24+1))."""
+        return qfx.Circuit.from_rows(self.rows, self.cols, self._template_gates, self._mats)
+
+
 def _circuit_with(template, gates_host):
-    """The template with its gate matrices replaced by the rows of gates_host ([n, 4] or
-    [n, 16]): 2x2 for a single-qubit gate, 4 diagonal entries for a diagonal two-qubit
-    gate (its first 4 values), 4x4 for a general one (16 values, rows of width 16 only)."""
-    c = copy.copy(template)
-    c.gates = []
-    for g, m in zip(template.gates, gates_host):
-        g2 = copy.copy(g)
-        if g.q1 < 0:
-            g2.mat = m[:4].reshape(2, 2).copy()
-        elif g.mat.size == 16:
-            if m.size != 16:
-                raise ValueError("a general (U4) gate needs gates rows of 16 entries")
-            g2.mat = m.reshape(4, 4).copy()
-        else:
-            g2.mat = m[:4].reshape(4).copy()
-        c.gates.append(g2)
-    return c
+    """The template with its gate matrices replaced by the rows of gates_host."""
+    width = gates_host.shape[1]
+    if width < 4:
+        raise ValueError("gates rows need at least 4 entries")
+    if width != 16 and any(g.q1 >= 0 and g.mat.size == 16 for g in template.gates):
+        raise ValueError("a general (U4) gate needs gates rows of 16 entries")
+    return _Rebuilt(template, gates_host[:, :16])
 
 
 def _make():
@@ -44,7 +63,7 @@ def _make():
         @staticmethod
         def forward(ctx, gates, template, x1, n_open: int = 0, open_sites=None, cuts=()):
             circ = _circuit_with(template, gates.detach().cpu().numpy())
-            plan = qfx.Plan(qfx.Circuit(circ), n_open=n_open, open_sites=open_sites, cuts=cuts)
+            plan = qfx.Plan(circ.compile(), n_open=n_open, open_sites=open_sites, cuts=cuts)
             ws = torch.empty(plan.workspace_bytes(1), dtype=torch.uint8, device=x1.device)
             amp = qfx.amplitudes(plan, x1, workspace=ws)
             ctx.plan = plan

@@ -207,29 +207,39 @@ int num_sms() {
   return n[dev] > 0 ? n[dev] : 1;
 }
 
-// Variants 0..9 keep their tile when its grid has more CTAs than there are SMs: two of them
-// share an SM, so up to twice as many run at once, and the fill tiles, with more reads of
-// shared memory per product, gain nothing (8 x 4096 columns, K = N = 64, 256 CTAs: 28.7 us
-// against 28.8; 65536 columns of K = 256, N = 16, 256 CTAs: 72 against 80).  Smaller grids
-// take the fill variant of the same row range (QFX_SIMT_FILL_VARIANTS) when it gives more
-// CTAs.  Both sum every output's k terms in the same order, so the choice never changes a
-// result.
+// Variants 0..9 keep their tile when its grid gives more than three CTAs to two SMs: two of
+// them share an SM, and the fill tiles, with more reads of shared memory per product, gain
+// nothing (8 x 4096 columns, K = N = 64, 256 CTAs: 28.7 us against 28.8; 65536 columns of
+// K = 256, N = 16, 256 CTAs: 72 against 80; but 208 CTAs, K = 1024, N = 512: 351 against 282).
+// On a smaller grid a tile's time is the latency of its k loop, the less the fewer products it
+// has: the step takes the first of the fill tiles below, in this order, that gives more CTAs
+// than SMs, or else the one that gives most (852 columns of K = 1024, N = 512: 345 us with 64 x
+// 128, 195 with 64 x 64, 135 with 16 x 128).  Every tile sums an output's k terms in the same
+// order, so the choice never changes a result.
 int fill_variant(int variant, int64_t N, int64_t J, int batch) {
-  static const int bm[10] = {128, 64, 32, 16, 8, 128, 64, 32, 16, 8};
-  static const int bj[10] = {64, 128, 256, 256, 512, 64, 128, 256, 256, 512};
-  static const int fill[10] = {20, 20, 21, 22, 23, 25, 25, 26, 27, 28};
-  static const int fbm[10] = {64, 64, 32, 16, 8, 64, 64, 32, 16, 8};
-  static const int fbj[10] = {64, 64, 128, 128, 256, 64, 64, 128, 128, 256};
+  struct Tile { int bm, bj; };
+  static const Tile base[5] = {{128, 64}, {64, 128}, {32, 256}, {16, 256}, {8, 512}};
+  static const Tile fill[5] = {{64, 64}, {32, 128}, {16, 128}, {8, 256}, {8, 128}};   // 20..24, 25..29
   if (variant < 0 || variant > 9 || batch < 1) return variant;
-  const int64_t blocks = ((N + bm[variant] - 1) / bm[variant]) * ((J + bj[variant] - 1) / bj[variant]) * batch;
-  if (blocks > (int64_t)num_sms()) return variant;
-  const int64_t fb = ((N + fbm[variant] - 1) / fbm[variant]) * ((J + fbj[variant] - 1) / fbj[variant]) * batch;
-  return fb > blocks ? fill[variant] : variant;
+  auto ctas = [&](const Tile& t) { return ((N + t.bm - 1) / t.bm) * ((J + t.bj - 1) / t.bj) * batch; };
+  const int64_t sms = num_sms();
+  int64_t most = ctas(base[variant % 5]);
+  if (2 * most > 3 * sms) return variant;
+  int best = variant;
+  for (int i = 0; i < 5; ++i) {
+    if (fill[i].bm > base[variant % 5].bm) continue;
+    const int64_t c = ctas(fill[i]);
+    if (c <= most) continue;
+    most = c;
+    best = 20 + i + (variant >= 5 ? 5 : 0);
+    if (c > sms) break;
+  }
+  return best;
 }
 
 bool simt_variant_valid(int variant, int64_t Sd) {
-  const bool jmode = (variant >= 0 && variant < 5) || (variant >= 20 && variant < 24);
-  const bool kmode = (variant >= 5 && variant < 10) || (variant >= 25 && variant < 29);
+  const bool jmode = (variant >= 0 && variant < 5) || (variant >= 20 && variant < 25);
+  const bool kmode = (variant >= 5 && variant < 10) || (variant >= 25 && variant < 30);
   return (jmode && Sd % 2 == 0) || kmode;
 }
 

@@ -296,6 +296,7 @@ struct TcArgs {
   int NHt;           // tiles along n per 128-row tile
   int64_t JT;        // 128-row tiles per item (256-row ones for pairs)
   int64_t tiles;     // total tiles (items x JT x NHt)
+  int sd_shift;      // log2 Sd where Sd is a power of two, else -1
   int withhold_s;    // test hook: never stream S, so the bounded waits expire
   int use_tma;       // pair tiles: producers read FP32 rows staged by tensor-map copies
   int stages, nbuf;  // pair tiles: operand stages and staging buffers
@@ -315,13 +316,30 @@ constexpr uint32_t kAlignPad = 128;
 constexpr int64_t kBand = 8;
 __device__ __forceinline__ void tile_coords(const TcArgs& a, int64_t t, int64_t& g, int64_t& jt,
                                             int64_t& nh) {
-  int64_t r, band;
-  divmod(t, a.JT * a.NHt, g, r);
-  divmod(r, kBand * a.JT, band, r);
-  const int64_t n0 = band * kBand;
-  const int64_t w = a.NHt - n0 < kBand ? a.NHt - n0 : kBand;
-  divmod(r, w, jt, r);
-  nh = n0 + r;
+  int64_t r = t, band;
+  g = 0;
+  if (a.tiles > a.JT * a.NHt) divmod(t, a.JT * a.NHt, g, r);
+  int64_t n0 = 0, w = a.NHt;
+  if (a.NHt > kBand) {
+    divmod(r, kBand * a.JT, band, r);
+    n0 = band * kBand;
+    w = a.NHt - n0 < kBand ? a.NHt - n0 : kBand;
+  }
+  jt = r;
+  nh = n0;
+  if (w > 1) {
+    divmod(r, w, jt, r);
+    nh = n0 + r;
+  }
+}
+// row index j = p * Sd + s
+__device__ __forceinline__ void split_row(const TcArgs& a, int64_t j, int64_t& p, int64_t& s) {
+  if (a.sd_shift >= 0) {
+    p = j >> a.sd_shift;
+    s = j & (a.Sd - 1);
+  } else {
+    divmod(j, a.Sd, p, s);
+  }
 }
 
 // ---- fast accumulation: one CTA per SM, one accumulator pair -------------------------
@@ -773,7 +791,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
           coords(t, g, jt, nh);
           const int64_t jg = jt * kRows + prow;
           inside = jg < a.J;
-          divmod(jg, a.Sd, p, sidx);
+          split_row(a, jg, p, sidx);
           src = a.B + g * a.b_stride + p * a.K * a.Sd + sidx + (int64_t)(kh * KH) * a.Sd;
         }
 #pragma unroll
@@ -844,7 +862,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
       for (int64_t t = pair0; t < a.tiles && ok; t += pairs) {
         int64_t g, jt, nh, p, sidx;
         coords(t, g, jt, nh);
-        divmod(jt * kRows, a.Sd, p, sidx);
+        split_row(a, jt * kRows, p, sidx);
         for (int it = 0; it < KT; ++it) {
           if (!mbar_wait(in_empty(in.i), in.pass ^ 1u, abort)) { ok = false; break; }
           mbar_arrive_tx(in_full(in.i), (uint32_t)CF::STAGE_IN);
@@ -921,11 +939,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
     // ..., AHEAD of them in registers before the first is stored
     constexpr int MOST = CF::NT_MAX / 16, AHEAD = 5, RING = AHEAD + 1;
     const int mine = a.Nt / 16;
-    const int NL = (int)a.NL;
+    const int N = (int)a.N, NL = (int)a.NL;
     const int64_t wrap = a.P * a.NL * a.Sd - (int64_t)NL * a.Sd;   // from the end of one nh to the next
     Ring acc;
     for (int64_t t = pair0; t < a.tiles; t += pairs) {
-      if (!__all_sync(0xffffffffu, mbar_wait(acc_full(acc.i), acc.pass, abort, 64))) break;
+      // addresses first, while the MMAs of the tile run
+      int64_t g, jt, nh, p, sidx;
+      coords(t, g, jt, nh);
+      const int64_t jg = jt * kRows + row;
+      const bool valid = jg < a.J;
+      split_row(a, jg, p, sidx);
+      float2* Cj = a.C + g * a.c_stride + p * a.NL * a.Sd + sidx;
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full(acc.i), acc.pass, abort))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t main0 = tmem + (uint32_t)(acc.i * 256) + lane_base;
       const uint32_t small0 = main0 + (uint32_t)(n_acc == 2 ? 2 * a.Nt : 256);
@@ -949,20 +974,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
 #pragma unroll
       for (int i = 0; i < AHEAD; ++i)
         if (i < mine) load(i, i);
-      int64_t g, jt, nh, p, sidx;
-      coords(t, g, jt, nh);
-      const int64_t jg = jt * kRows + row;
-      const bool valid = jg < a.J;
-      divmod(jg, a.Sd, p, sidx);
-      float2* Cj = a.C + g * a.c_stride + p * a.NL * a.Sd + sidx;
 #pragma unroll
       for (int i = 0; i < MOST; ++i) {
         if (i + AHEAD < MOST && i + AHEAD < mine) load(i + AHEAD, (i + AHEAD) % RING);
         if (i < mine && valid) {
           const int buf = i % RING;
-          // one division per chunk, then step along n with a carry into nh
+          // columns n0 .. n0 + 7 of S: one division (none where n does not split) and, where the
+          // chunk crosses from one nh to the next, a carry
           const int n0 = (int)nh * a.Nt + (half + 2 * i) * 8;
-          const int nh0 = n0 / NL;
+          const int nh0 = NL == N ? 0 : n0 / NL;
           int left = (nh0 + 1) * NL - n0;   // columns to the end of this nh
           float2* dst = Cj + nh0 * wrap + (int64_t)n0 * a.Sd;
           if (a.beta) {   // a chunk of a long contraction: add into C
@@ -980,11 +1000,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
 #pragma unroll
             for (int e = 0; e < 8; ++e) { vr[buf][e] += o[e].x; vi[buf][e] += o[e].y; }
           }
+          if (left >= 8) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            *dst = make_float2(vr[buf][e], vi[buf][e]);
-            dst += a.Sd;
-            if (--left == 0) { left = NL; dst += wrap; }
+            for (int e = 0; e < 8; ++e) {
+              *dst = make_float2(vr[buf][e], vi[buf][e]);
+              dst += a.Sd;
+            }
+          } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              *dst = make_float2(vr[buf][e], vi[buf][e]);
+              dst += a.Sd;
+              if (--left == 0) { left = NL; dst += wrap; }
+            }
           }
         }
       }
@@ -1132,6 +1160,9 @@ int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, in
   const int rows = fast ? kRows : 2 * kRows;
   a.JT = (a.J + rows - 1) / rows;
   a.tiles = (int64_t)batch * a.JT * a.NHt;
+  a.sd_shift = -1;
+  for (int b = 0; b < 62; ++b)
+    if (Sd == int64_t(1) << b) a.sd_shift = b;
   a.withhold_s = withhold;
   a.beta = beta;
   if (fast) {

@@ -319,19 +319,19 @@ __device__ __forceinline__ void cgemm_tile(const StepArgs& a, int64_t tile, int6
   X(8, 16, 256, 4, 4, true)         \
   X(9, 8, 512, 4, 4, true)
 
-// Fill variants: tiles with a half or a quarter of the outputs per CTA, for grids that the
-// tiles above would leave with fewer CTAs than two per SM (fill_variant picks them at launch
-// time; the batch scheduler keeps 0..9).  Variants 0, 1, 2, 3, 4 map to 20, 20, 21, 22, 23
-// and 5..9 to 25, 25, 26, 27, 28.
+// Fill variants: smaller tiles for grids that the tiles above would leave with fewer CTAs than
+// SMs (fill_variant picks them at launch time; the batch scheduler keeps 0..9).
 #define QFX_SIMT_FILL_VARIANTS(X)   \
   X(20, 64, 64, 4, 4, false)        \
   X(21, 32, 128, 4, 4, false)       \
   X(22, 16, 128, 2, 4, false)       \
   X(23, 8, 256, 2, 4, false)        \
+  X(24, 8, 128, 2, 2, false)        \
   X(25, 64, 64, 4, 4, true)         \
   X(26, 32, 128, 4, 4, true)        \
   X(27, 16, 128, 2, 4, true)        \
-  X(28, 8, 256, 2, 4, true)
+  X(28, 8, 256, 2, 4, true)         \
+  X(29, 8, 128, 2, 2, true)
 
 }  // namespace simt
 }  // namespace qfx

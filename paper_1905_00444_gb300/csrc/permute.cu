@@ -16,7 +16,6 @@
 #include <algorithm>
 #include <cstring>
 
-#include "launch.cuh"
 #include "ptx_async.cuh"
 #include "qfx_internal.h"
 
@@ -49,11 +48,9 @@ struct PermArgs {
 // divisions) and steps an odometer through the rest.
 constexpr int kRowChunk = 4096;
 constexpr int kMaxChunkRows = kRowChunk / 2 + 2;   // D >= 2 for this kernel
-__global__ void __launch_bounds__(256) permute_rows_kernel(const float2* in,
-                                                           float2* out,
+__global__ void __launch_bounds__(256) permute_rows_kernel(const float2* __restrict__ in,
+                                                           float2* __restrict__ out,
                                                            const PermArgs a, int64_t total) {
-  launch_next();
-  launch_wait();
   __shared__ int64_t rowoff[kMaxChunkRows];
   const int64_t D = a.dim[a.rank - 1];
   const int64_t base = (int64_t)blockIdx.x * kRowChunk;
@@ -100,11 +97,9 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const float2* in,
 }
 
 // Rows of one element (or longer than 2^30): the mixed-radix divisions stay per element.
-__global__ void __launch_bounds__(256) permute_short_rows_kernel(const float2* in,
-                                                                 float2* out,
+__global__ void __launch_bounds__(256) permute_short_rows_kernel(const float2* __restrict__ in,
+                                                                 float2* __restrict__ out,
                                                                  const PermArgs a, int64_t total) {
-  launch_next();
-  launch_wait();
   const int64_t D = a.dim[a.rank - 1];
   const int64_t o = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (o >= total) return;
@@ -122,11 +117,9 @@ __global__ void __launch_bounds__(256) permute_short_rows_kernel(const float2* i
 // A block handles kTileBatch consecutive batch coordinates of one (a, b) tile position,
 // stepping the batch odometer instead of decomposing every tile's index.
 constexpr int kTileBatch = 8;
-__global__ void __launch_bounds__(256) permute_tile_kernel(const float2* in,
-                                                           float2* out,
+__global__ void __launch_bounds__(256) permute_tile_kernel(const float2* __restrict__ in,
+                                                           float2* __restrict__ out,
                                                            const PermArgs a, int64_t batch) {
-  launch_next();
-  launch_wait();
   __shared__ float2 tile[32][33];
   __shared__ int64_t offa[32];
   const int64_t per = a.tiles_a * a.tiles_b;
@@ -245,7 +238,7 @@ __device__ __forceinline__ void perm_issue(const PermTma& a, const CUtensorMap* 
 // buffer once its 128 consumers have released it.  Every wait is bounded; a timeout sets
 // the status word and makes the other roles give up too.
 template <int TA, int NB>
-__global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float2* out,
+__global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float2* __restrict__ out,
                                                           const __grid_constant__ CUtensorMap map) {
   constexpr int TB = 16;
   const int TILE = TB * TA * 8 * a.BZ, UNITS = 8 * (TA / 16) * a.BZ;
@@ -265,8 +258,6 @@ __global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float
     mbar_init_fence();
   }
   __syncthreads();
-  launch_next();
-  launch_wait();
   volatile int* abort = &abort_flag;
   auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
     if (mbar_try(bar, parity)) return true;
@@ -423,7 +414,8 @@ int launch_perm_tma(const PermTma& a, const CUtensorMap& map, float2* out, cudaS
   per_sm = per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm;
   const int64_t want = (int64_t)(sms > 0 ? sms : 1) * per_sm;
   const unsigned grid = (unsigned)(a.total < want ? a.total : want);
-  return (int)launch_early(permute_tma_kernel<TA, NB>, dim3(grid), dim3(160), smem, st, a, out, map);
+  permute_tma_kernel<TA, NB><<<grid, 160, smem, st>>>(a, out, map);
+  return (int)cudaGetLastError();
 }
 }  // namespace
 
@@ -458,16 +450,15 @@ int launch_permute(const void* in, void* out, int rank, const int64_t* shape,
   cudaStream_t st = (cudaStream_t)stream;
   const float2* src = (const float2*)in;
   float2* dst = (float2*)out;
-  cudaError_t e = cudaSuccess;
   if (a.istr[fr - 1] == 1) {
     if (a.dim[fr - 1] >= 2 && a.dim[fr - 1] < (int64_t(1) << 30)) {
       const int64_t blocks = (total + kRowChunk - 1) / kRowChunk;
       if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
-      e = launch_early(permute_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, st, src, dst, a, total);
+      permute_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dst, a, total);
     } else {
       const int64_t blocks = (total + 255) / 256;
       if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
-      e = launch_early(permute_short_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, st, src, dst, a, total);
+      permute_short_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dst, a, total);
     }
   } else {
     a.la = fr - 1;
@@ -504,10 +495,10 @@ int launch_permute(const void* in, void* out, int rank, const int64_t* shape,
     const int64_t batch = total / (a.da * a.dim[a.lb]);
     const int64_t blocks = ((batch + kTileBatch - 1) / kTileBatch) * a.tiles_a * a.tiles_b;
     if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
-    e = launch_early(permute_tile_kernel, dim3((unsigned)blocks), dim3(256), 0, st, src, dst, a, batch);
+    permute_tile_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dst, a, batch);
   }
   count_launch();
-  return (int)e;
+  return (int)cudaGetLastError();
 }
 
 int perm_take_status() {

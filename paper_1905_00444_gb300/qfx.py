@@ -10,6 +10,8 @@ import os
 import re
 from typing import Iterable, List, Optional, Sequence
 
+import numpy as np
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libqfx.so")
 HEADER = os.path.join(os.path.dirname(HERE), "include", "qfx.h")
@@ -143,6 +145,33 @@ def launch_count() -> int:
     return int(lib.qfx_launch_count())
 
 
+# struct Gate as a numpy record, so that tables of gates are filled by column
+GATE_DTYPE = np.dtype([("layer", np.int32), ("q0", np.int32), ("q1", np.int32), ("kind", np.int32),
+                       ("mat", np.complex128, 16)])
+assert GATE_DTYPE.itemsize == C.sizeof(Gate)
+
+
+def gate_table(gates, mats):
+    """The ABI's gate records for `gates` (their .layer, .q0, .q1 and .kind) with the matrix
+    entries of `mats`: one sequence of up to 16 entries per gate, or one array of them all
+    [n_gates, width].  A gate's entries past its own are zero."""
+    table = np.zeros(max(1, len(gates)), dtype=GATE_DTYPE)
+    if not gates:
+        return table
+    table["layer"], table["q0"], table["q1"], table["kind"] = zip(
+        *[(g.layer, g.q0, g.q1, g.kind) for g in gates])
+    if isinstance(mats, np.ndarray):
+        table["mat"][:, :mats.shape[1]] = mats
+        return table
+    sizes = np.array([len(m) for m in mats])
+    if sizes.max() > 16:
+        raise IndexError("a gate has at most 16 matrix entries")
+    for size in np.unique(sizes):
+        rows = np.flatnonzero(sizes == size)
+        table["mat"][rows, :size] = np.array([mats[i] for i in rows])
+    return table
+
+
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         import torch
@@ -163,17 +192,26 @@ class Circuit:
             self.n_gates = sum(1 for ln in text.splitlines()
                                if ln.split("#")[0].strip() and not ln.strip().startswith("grid"))
         else:
-            arr = (Gate * max(1, len(src.gates)))()
-            for i, g in enumerate(src.gates):
-                arr[i].layer, arr[i].q0, arr[i].q1, arr[i].kind = g.layer, g.q0, g.q1, g.kind
-                flat = list(g.mat.reshape(-1))
-                for j, v in enumerate(flat):
-                    arr[i].mat[2 * j] = float(v.real)
-                    arr[i].mat[2 * j + 1] = float(v.imag)
-            _check(lib.qfx_circuit_create(src.rows, src.cols, arr, len(src.gates), C.byref(h)))
-            self.rows, self.cols = src.rows, src.cols
-            self.n_gates = len(src.gates)
+            self._create(src.rows, src.cols, src.gates,
+                         [np.asarray(g.mat).reshape(-1) for g in src.gates], h)
         self._h = h
+
+    def _create(self, rows, cols, gates, mats, h):
+        table = gate_table(gates, mats)
+        _check(lib.qfx_circuit_create(rows, cols, table.ctypes.data_as(C.POINTER(Gate)), len(gates), C.byref(h)))
+        self.rows, self.cols = rows, cols
+        self.n_gates = len(gates)
+
+    @classmethod
+    def from_rows(cls, rows, cols, gates, mats):
+        """A circuit of `gates` (.layer, .q0, .q1, .kind) whose matrices are the rows of the
+        array `mats` [n, 4 or 16] (as many gates as there are rows)."""
+        self = cls.__new__(cls)
+        h = C.c_void_p()
+        n = min(len(gates), len(mats))
+        self._create(rows, cols, gates[:n], mats[:n], h)
+        self._h = h
+        return self
 
     def __del__(self):
         if getattr(self, "_h", None):
