@@ -656,6 +656,15 @@ template <int N>
 __device__ __forceinline__ void reg_take() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
+// Barrier of the 8 producer warps; true for all of them where `p` holds for any.
+__device__ __forceinline__ bool producers_any(bool p) {
+  uint32_t r;
+  __syncwarp();
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, 1, 256, p;\nselp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r) : "r"((uint32_t)p) : "memory");
+  return r != 0;
+}
 // Registers per thread of the roles' warpgroups; the launch gives each of the five 96.
 constexpr int kRegLaunch = 96, kRegProd = 72, kRegCtl = 48, kRegEpi = 144;
 static_assert(2 * kRegProd + kRegCtl + 2 * kRegEpi <= 5 * kRegLaunch, "the roles share the launch's registers");
@@ -696,7 +705,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   if (tid == 0) {
     abort_flag = 0;
     for (int s = 0; s < stages; ++s) {
-      mbar_init(full(s), 18);        // 8 producer warps and the site copies of each CTA
+      mbar_init(full(s), 4);         // the producers and the site copies of each CTA
       mbar_init(fullS(s), 1);
       mbar_init(empty(s), 1);
     }
@@ -707,7 +716,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
     mbar_init(done, 1);
     for (int b = 0; b < nbuf; ++b) {
       mbar_init(in_full(b), 1);
-      mbar_init(in_empty(b), 8);
+      mbar_init(in_empty(b), 1);
     }
     mbar_init_fence();
   }
@@ -735,24 +744,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   if (warp < 8) {
     // ---- producers: split 128 rows of B per k-stage into term planes -------------------
     reg_release<kRegProd>();
-    // Two threads share a row, each half of its k.  The proxy fence is the largest part of a
-    // stage's latency, so there is one for both what it orders: the operand planes before the
-    // MMAs that read them, and the reads of the staging buffer before the copy that reuses it.
+    // Two threads share a row, each half of its k.  A barrier among the producers collects a
+    // stage's reads and writes, and one thread's proxy fence behind it orders them all: the
+    // operand planes before the MMAs that read them, the staging buffer's reads before the copy
+    // that reuses it.  A fence in every warp held up the SM's other memory instructions, the
+    // epilogue's stores above all (K = N = 256 over 2^19 columns, TF32x3: 1.02 -> 0.91 ms).
     constexpr int KH = KS / 2;
     const int prow = tid & (kRows - 1), kh = tid >> 7;
     const int64_t n_stages = pair0 < a.tiles ? ((a.tiles - pair0 + pairs - 1) / pairs) * KT : 0;
     Ring op;                    // operand stages
     float re[SUB][KH], im[SUB][KH];
-    auto put = [&]() -> bool {   // re, im into the next operand stage; false on a timeout
-      if (!__all_sync(0xffffffffu, mbar_wait(empty(op.i), op.pass ^ 1u, abort))) return false;
-      char* st = sA + op.i * CF::STAGE_A;
+    // re, im into the next operand stage, unless a wait ran out (`ok` false): then, at once for
+    // all producers, false
+    auto put = [&](bool ok) -> bool {
+      if (ok) ok = mbar_wait(empty(op.i), op.pass ^ 1u, abort);
+      if (ok) {
+        char* st = sA + op.i * CF::STAGE_A;
 #pragma unroll
-      for (int u = 0; u < SUB; ++u) {
-        store_half_terms<MODE>(st + u * CF::PLANES * kPlaneA, prow, kh, re[u]);
-        store_half_terms<MODE>(st + (u * CF::PLANES + TERMS) * kPlaneA, prow, kh, im[u]);
+        for (int u = 0; u < SUB; ++u) {
+          store_half_terms<MODE>(st + u * CF::PLANES * kPlaneA, prow, kh, re[u]);
+          store_half_terms<MODE>(st + (u * CF::PLANES + TERMS) * kPlaneA, prow, kh, im[u]);
+        }
       }
-      fence_async_smem();
-      __syncwarp();
+      if (producers_any(!ok)) return false;
+      if (tid == 0) {
+        fence_async_smem();
+        mbar_arrive_leader(full(op.i));
+      }
+      op.step(stages);
       return true;
     };
     if (a.use_tma) {
@@ -760,22 +779,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
       const int in_ofs = (ps * SUB * KS + kh * KH) * a.box_s + ss;
       Ring in;
       for (int64_t q = 0; q < n_stages; ++q) {
-        if (!__all_sync(0xffffffffu, mbar_wait(in_full(in.i), in.pass, abort))) break;
-        const float2* src = reinterpret_cast<const float2*>(sIn + in.i * CF::STAGE_IN) + in_ofs;
+        const bool ok = mbar_wait(in_full(in.i), in.pass, abort);
+        if (ok) {
+          const float2* src = reinterpret_cast<const float2*>(sIn + in.i * CF::STAGE_IN) + in_ofs;
 #pragma unroll
-        for (int u = 0; u < SUB; ++u)
+          for (int u = 0; u < SUB; ++u)
 #pragma unroll
-          for (int kk = 0; kk < KH; ++kk) {   // rows past K arrive as zeros
-            const float2 v = src[(u * KS + kk) * a.box_s];
-            re[u][kk] = v.x;
-            im[u][kk] = v.y;
-          }
-        if (!put()) break;
-        if (lane == 0) {
-          mbar_arrive_leader(full(op.i));
-          mbar_arrive(in_empty(in.i));
+            for (int kk = 0; kk < KH; ++kk) {   // rows past K arrive as zeros
+              const float2 v = src[(u * KS + kk) * a.box_s];
+              re[u][kk] = v.x;
+              im[u][kk] = v.y;
+            }
         }
-        op.step(stages);
+        if (!put(ok)) break;
+        if (tid == 0) mbar_arrive(in_empty(in.i));
         in.step(nbuf);
       }
     } else {
@@ -809,9 +826,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
 #pragma unroll
           for (int kk = 0; kk < KH; ++kk) { re[u][kk] = nxt[u][kk].x; im[u][kk] = nxt[u][kk].y; }
         if (q + 1 < n_stages) fetch();
-        if (!put()) break;
-        if (lane == 0) mbar_arrive_leader(full(op.i));
-        op.step(stages);
+        if (!put(true)) break;
       }
     }
   } else if (warp < 12) {
