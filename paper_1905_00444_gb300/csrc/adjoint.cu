@@ -746,11 +746,8 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
 
   for (int64_t item = 0; item < n_items; ++item) {
     const int64_t b = item % n_batch, sid = slice_begin + item / n_batch;
-    e = cudaMemsetAsync(hdr, 0, (size_t)n * 8 + 16, st);
-    if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes_backward: header");
-    int err = launch_fold(t, n, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch, slice_begin,
+    int err = launch_sites(t, n, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch, slice_begin,
                           item, 1, hdr, 0, sites, 0, 0, st);
-    if (!err) err = launch_scale(t, n, max_site, 1, hdr, 0, sites, 0, 0, st);
     if (err) return cuda_fail(err, "qfx_amplitudes_backward: fold");
     if (ctab.count > 0) {
       err = (int)launch_early(conj_transpose_kernel, dim3((unsigned)conj_tiles, (unsigned)ctab.count), dim3(kT), 0, st,

@@ -603,15 +603,15 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
 //   176 KB = 1375 clk at 128 B/clk against 1638 clk of MMA at the measured rate,
 // where a single CTA moves 236 KB = 1844 clk.  Measured against such a single CTA (K = N = 256,
 // 2^19 columns): one cool launch takes 0.82 ms (0.83 of the tensor probe) against 0.98; run
-// for seconds both are held by the 1400 W limit, 1.02 against 1.07 ms for BF16x3 and 0.97
-// against 1.02 for TF32x3; BF16x2 at K = N = 1024 over 2^15 columns went from 0.67 to 0.53 ms.
+// for seconds both are held by the 1400 W limit, 0.96 against 1.07 ms for BF16x3 and 0.91
+// against 1.02 for TF32x3; BF16x2 at K = N = 1024 over 2^15 columns went from 0.67 to 0.50 ms.
 //
 // With 4 Nt <= 256 the accumulators of two tiles fit the TMEM (the halves of its 512
 // columns): the MMAs of a tile run while the epilogue stores the one before.  At Nt = 128
 // they take turns, and the MMAs wait until the epilogue has read them.  Its stores back up
 // (100 clk for each of 256 bytes, with every SM storing at once), so it reads ahead of them:
-// with registers taken over from the other roles it holds 6 chunks of 8 columns beside the one
-// it stores, and hands the TMEM back after the second of its 8 chunks.
+// with registers taken over from the other roles it holds 5 chunks of 8 columns beside the one
+// it stores, and hands the TMEM back after the third of its 8 chunks.
 //
 // Roles, in each CTA on its own 128 rows: warps 0-7 producers, 8 TMEM owner and MMA issuer, 9
 // site stream, 10 tensor-map copies, 12-19 epilogue (two per TMEM lane quarter).  CTA 0 (the
@@ -623,10 +623,11 @@ template <int MODE>
 struct PairCfg {
   using M_ = Mode<MODE>;
   static constexpr int NT_MAX = 128;
-  // k-steps (of one MMA per product) in an operand stage: the fences, arrivals and waits of a
+  // k-steps (of one MMA per product) in an operand stage: the fence, arrivals and waits of a
   // stage cost its roles 500 to 800 clk, which the 6 MMAs of a two-term k-step (819 clk) barely
   // cover.  Two k-steps of TF32 take the bytes of one of BF16 (K = N = 256 over 2^19 columns:
-  // 984 -> 903 us); two of BF16x2 leave room for two stages only (490 -> 515 us at K = 1024).
+  // 984 -> 903 us when it was chosen); two of BF16x2 leave room for two stages only (490 -> 515
+  // us at K = 1024).
   static constexpr int SUB = M_::KS == 8 ? 2 : 1;
   static constexpr int PLANES = 2 * M_::TERMS;              // planes of each operand per k-step
   static constexpr int STAGE_A = SUB * PLANES * kPlaneA;

@@ -2,7 +2,8 @@
 // (programmatic dependent launch).  Such a kernel sets itself up and then waits, before it
 // touches any global memory, until the kernels ahead of it have completed and their writes
 // are visible; a kernel that lets its successor start early says so once its own blocks are
-// running.  Between the small kernels of a sweep this hides most of the launch latency.
+// running.  Between the small kernels of a sweep this hides most of the launch latency (all
+// amplitudes of 4x4x(1+16+1), 21 calls: 155 -> 122 us).
 // Such a kernel declares inputs that an earlier one writes without __restrict__: loads that the
 // compiler takes for invariant may move above the wait.
 #pragma once

@@ -187,13 +187,12 @@ qfx_status fail(qfx_status st, const std::string& msg);
 qfx_status cuda_fail(int err, const char* what);
 
 // kernels (implemented in .cu files); all return 0 or a cudaError_t value
-int launch_fold(const DeviceTables& t, int n_sites, int64_t max_site_size, int n_cuts,
-                const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
-                int64_t item0, int items, char* hdr, uint64_t hdr_stride, char* itemsp,
-                uint64_t item_bytes, uint64_t sites_off, void* stream);
-int launch_scale(const DeviceTables& t, int n_sites, int64_t max_site_size, int items,
-                 char* hdr, uint64_t hdr_stride, char* itemsp, uint64_t item_bytes,
-                 uint64_t sites_off, void* stream);
+// folds the site tensors of `items` work items and scales each by a power of two, whose
+// exponent goes to the item's header
+int launch_sites(const DeviceTables& t, int n_sites, int64_t max_site_size, int n_cuts,
+                 const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
+                 int64_t item0, int items, char* hdr, uint64_t hdr_stride, char* itemsp,
+                 uint64_t item_bytes, uint64_t sites_off, void* stream);
 int launch_accumulate(const DeviceTables& t, int n_sites, int n_open, int64_t n_batch,
                       int64_t item0, int items, const char* hdr, uint64_t hdr_stride,
                       const char* itemsp, uint64_t item_bytes, uint64_t final_off, double* out,

@@ -214,20 +214,14 @@ static qfx_status exec_tree(const qfx_plan* p, const DeviceTables& t, const uint
   for (const auto& fs : p->sites) max_site = std::max(max_site, fs.size);
   char* hdr_base = (char*)workspace;
   char* items = hdr_base + align256((uint64_t)G * hdr);
-  cudaError_t e = cudaMemsetAsync(out, 0, (size_t)(n_batch << n_open) * 16, st);
-  if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes: clearing out");
   for (int64_t item0 = 0; item0 < n_items; item0 += G) {
     const int g = (int)std::min<int64_t>(G, n_items - item0);
-    e = cudaMemsetAsync(hdr_base, 0, (size_t)g * hdr, st);
-    if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes: clearing header");
     int slot;
     profile_begin(st, &slot);
-    int err = launch_fold(t, p->n, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch,
+    int err = launch_sites(t, p->n, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch,
                           slice_begin, item0, g, hdr_base, hdr, items, ib, L.sites, st);
     profile_end(st, slot, -1, 0, 1, 0.0, 0.0);
-    if (err) return cuda_fail(err, "fold kernel");
-    err = launch_scale(t, p->n, max_site, g, hdr_base, hdr, items, ib, L.sites, st);
-    if (err) return cuda_fail(err, "scale kernel");
+    if (err) return cuda_fail(err, "fold and scale kernels");
     for (size_t i = 0; i < p->tree.size(); ++i) {
       const TreeNode& nd = p->tree[i];
       for (int gi = 0; gi < g && (nd.permA || nd.permB); ++gi) {
@@ -310,20 +304,14 @@ qfx_status exec_amplitudes(const qfx_plan* p, const DeviceTables& t, const uint6
   const uint64_t site0 = L.sites + (uint64_t)p->sites[p->steps[0].site].offset * 8;
   const uint64_t final_off = nsteps == 1 ? site0 : ((nsteps - 1) % 2 ? L.buf1 : L.buf0);
 
-  cudaError_t e = cudaMemsetAsync(out, 0, (size_t)(n_batch << n_open) * 16, st);
-  if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes: clearing out");
   for (int64_t item0 = 0; item0 < n_items; item0 += G) {
     const int g = (int)std::min<int64_t>(G, n_items - item0);
-    e = cudaMemsetAsync(hdr_base, 0, (size_t)g * hdr, st);
-    if (e != cudaSuccess) return cuda_fail(e, "qfx_amplitudes: clearing header");
     int slot;
     profile_begin(st, &slot);
-    int err = launch_fold(t, n_sites, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch,
+    int err = launch_sites(t, n_sites, max_site, (int)p->cut_dev.size(), x1, p->x1_words, n_batch,
                           slice_begin, item0, g, hdr_base, hdr, items, ib, L.sites, st);
     profile_end(st, slot, -1, 0, 1, 0.0, 0.0);
-    if (err) return cuda_fail(err, "fold kernel");
-    err = launch_scale(t, n_sites, max_site, g, hdr_base, hdr, items, ib, L.sites, st);
-    if (err) return cuda_fail(err, "scale kernel");
+    if (err) return cuda_fail(err, "fold and scale kernels");
     for (int i = 1; i < nsteps; ++i) {
       const Step& sp = p->steps[i];
       const char* S = items + L.sites + (uint64_t)p->sites[sp.site].offset * 8;
