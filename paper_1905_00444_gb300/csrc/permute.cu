@@ -7,7 +7,7 @@
 //   x BZ (consecutive values of one more axis) elements arrive by tensor-map copies with
 //   128-byte swizzle into a ring of shared buffers; each warp instruction then reads 16
 //   consecutive la by 2 consecutive lb (conflict-free under the swizzle) and writes two
-//   128-byte output segments.  The input is viewed as a 5-D tensor: lb, la, and the
+//   128-byte output segments; short output runs are lengthened by the axis next to la.  The input is viewed as a 5-D tensor: lb, la, and the
 //   other axes merged into at most three runs that are contiguous in the input.
 // - Otherwise a 32 x 32 tile goes through shared memory with plain loads, each block
 //   walking 8 consecutive batch coordinates.
@@ -185,9 +185,10 @@ struct PermTma {
   int64_t segE[3];          // run extents (coordinates 2..4 of the tensor map)
   int seg_n[3];             // axes per run, innermost first
   int64_t ax_dim[kMaxRank], ax_ostr[kMaxRank];   // the runs' axes, run by run
-  int BZ;                   // box extent along run 0 (divides its innermost axis)
-  int64_t tiles_z;          // segE[0] / BZ (1 if there is no run)
-  int64_t ostr_z;           // output stride of run 0's innermost axis
+  int bx[3];                // box extent along each run (divides its innermost axis)
+  int BZ, BY;               // box extents of the z run and of the run of the output axis next to la
+  int y_outer;              // the y run is a later (slower) box dimension than the z run
+  int64_t ostr_z, ostr_y;   // output strides of those runs' innermost axes
   unsigned long long wait_ns;   // limit of every bounded wait
   int withhold;             // test hook: issue no copies (every consumer's wait runs out)
 };
@@ -211,12 +212,11 @@ __device__ __forceinline__ void perm_issue(const PermTma& a, const CUtensorMap* 
   int64_t bi = r / a.tiles_b;
   int z[3] = {0, 0, 0};
   int64_t obase = ta * TA + tb * TB * a.ostr_b;
-  for (int g = a.nseg - 1; g >= 1; --g) {   // run 0 most significant
-    const int64_t zg = bi % a.segE[g];
-    bi /= a.segE[g];
-    z[g] = (int)zg;
+  for (int g = a.nseg - 1; g >= 0; --g) {   // run 0 most significant; each advances a box at a time
+    const int64_t E = a.segE[g] / a.bx[g], zg = bi % E;
+    bi /= E;
+    z[g] = (int)(zg * a.bx[g]);
   }
-  if (a.nseg > 0) z[0] = (int)(bi * a.BZ);  // run 0 advances a box of BZ at a time
   int ax = 0;
   for (int g = 0; g < a.nseg; ++g) {
     int64_t zg = z[g];
@@ -230,7 +230,7 @@ __device__ __forceinline__ void perm_issue(const PermTma& a, const CUtensorMap* 
   const int64_t ra = a.Da - ta * TA, rb = a.Db - tb * TB;
   meta->na = (int)(ra < TA ? ra : TA);
   meta->nb = (int)(rb < TB ? rb : TB);
-  mbar_arrive_tx(bar, (uint32_t)(TB * TA * a.BZ * 8));
+  mbar_arrive_tx(bar, (uint32_t)(TB * TA * a.BZ * a.BY * 8));
   tma_load_5d(dst, map, (int)(tb * TB), (int)(ta * TA), z[0], z[1], z[2], bar);
 }
 
@@ -241,7 +241,8 @@ template <int TA, int NB>
 __global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float2* __restrict__ out,
                                                           const __grid_constant__ CUtensorMap map) {
   constexpr int TB = 16;
-  const int TILE = TB * TA * 8 * a.BZ, UNITS = 8 * (TA / 16) * a.BZ;
+  const int TILE = TB * TA * 8 * a.BZ * a.BY, UNITS = 8 * (TA / 16) * a.BZ * a.BY;
+  const int by_shift = 31 - __clz(a.BY);   // BY is a power of two
   extern __shared__ char smem_raw[];
   // 128-byte swizzled boxes must start on 1024-byte boundaries
   char* buf = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -301,11 +302,14 @@ __global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float
     const TileMeta m = meta[b];
     const char* tile = buf + b * TILE;
     for (int u = warp; u < UNITS; u += 4) {
-      const int c = u & 7, iz = (u >> 3) / (TA / 16), ia = ((u >> 3) % (TA / 16)) * 16 + ia_lo, ib = 2 * c + h;
-      // row (iz, ia) of the box is 128 bytes of lb; its 16-byte chunk c sits at
-      // c ^ (row mod 8), and row mod 8 = ia mod 8 since TA is a multiple of 8
-      const float2 v = *reinterpret_cast<const float2*>(tile + (iz * TA + ia) * 128 + ((c ^ (ia & 7)) << 4) + h * 8);
-      if (ia < m.na && ib < m.nb) out[m.obase + iz * a.ostr_z + ia + (int64_t)ib * a.ostr_b] = v;
+      // iy fastest: neighbouring warps write neighbouring lines of an output run
+      const int iy = u & (a.BY - 1), w = u >> by_shift, c = w & 7;
+      const int iz = (w >> 3) / (TA / 16), ia = ((w >> 3) % (TA / 16)) * 16 + ia_lo, ib = 2 * c + h;
+      const int row = (a.y_outer ? iy * a.BZ + iz : iz * a.BY + iy) * TA + ia;
+      // a row of the box is 128 bytes of lb; its 16-byte chunk c sits at c ^ (row mod 8), and
+      // row mod 8 = ia mod 8 since TA is a multiple of 8
+      const float2 v = *reinterpret_cast<const float2*>(tile + row * 128 + ((c ^ (ia & 7)) << 4) + h * 8);
+      if (ia < m.na && ib < m.nb) out[m.obase + iy * a.ostr_y + iz * a.ostr_z + ia + (int64_t)ib * a.ostr_b] = v;
     }
     // the next copy into this buffer goes through the async proxy: order the reads first
     fence_async_smem();
@@ -330,47 +334,84 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   a.Da = Da;
   a.Db = Db;
   a.ostr_b = f.ostr[lb];
-  int64_t segS[3] = {1, 1, 1};
-  int ax = 0;
-  for (int i = 0; i < n;) {
-    if (a.nseg == 3) return false;
-    int j = i;   // run [i, j]: each next axis sits right inside the previous one in memory
-    while (j + 1 < n && f.istr[order[j]] == f.istr[order[j + 1]] * f.dim[order[j + 1]]) ++j;
-    int64_t E = 1;
-    for (int q = j; q >= i; --q) {   // innermost first
-      a.ax_dim[ax] = f.dim[order[q]];
-      a.ax_ostr[ax] = f.ostr[order[q]];
-      ++ax;
-      E *= f.dim[order[q]];
-    }
-    if (E > 0x7fffffff) return false;
-    a.segE[a.nseg] = E;
-    a.seg_n[a.nseg] = j - i + 1;
-    segS[a.nseg] = f.istr[order[j]];
-    ++a.nseg;
-    i = j + 1;
-  }
-  // strides of map dimensions 1..4 in bytes must be multiples of 16
-  if ((f.istr[la] & 1) || (a.nseg > 0 && (segS[0] & 1)) || (a.nseg > 1 && (segS[1] & 1)) ||
-      (a.nseg > 2 && (segS[2] & 1)))
-    return false;
   const int TA = Da >= 64 ? 64 : Da >= 32 ? 32 : 16;
   a.tiles_a = (Da + TA - 1) / TA;
   a.tiles_b = (Db + 15) / 16;
-  // boxes of 8 KB or more: BZ values of run 0's innermost axis (a divisor of its extent)
-  a.BZ = 1;
-  a.ostr_z = 0;
-  if (a.nseg > 0) {
-    const int want = 64 / TA;   // 1, 2 or 4 ... up to 8 for TA = 16
-    const int64_t d0 = a.ax_dim[0];   // run 0's innermost axis
-    int bz = 1;
-    while (bz * 2 <= (TA == 16 ? 8 : want) && d0 % (bz * 2) == 0) bz *= 2;
-    a.BZ = bz;
-    a.ostr_z = a.ax_ostr[0];
+  int64_t segS[3] = {1, 1, 1};
+  // cuts the other axes into runs, with axis `alone` (if any) a run of its own; false where
+  // there are more than three or the map's strides (dimensions 1..4, in bytes) are not
+  // multiples of 16
+  auto cut_runs = [&](int alone, int* alone_run) {
+    a.nseg = 0;
+    *alone_run = -1;
+    int ax = 0;
+    for (int i = 0; i < n;) {
+      if (a.nseg == 3) return false;
+      int j = i;   // run [i, j]: each next axis sits right inside the previous one in memory
+      while (j + 1 < n && f.istr[order[j]] == f.istr[order[j + 1]] * f.dim[order[j + 1]] && order[j] != alone &&
+             order[j + 1] != alone)
+        ++j;
+      int64_t E = 1;
+      for (int q = j; q >= i; --q) {   // innermost first
+        a.ax_dim[ax] = f.dim[order[q]];
+        a.ax_ostr[ax] = f.ostr[order[q]];
+        ++ax;
+        E *= f.dim[order[q]];
+      }
+      if (E > 0x7fffffff) return false;
+      if (order[i] == alone) *alone_run = a.nseg;
+      a.segE[a.nseg] = E;
+      a.seg_n[a.nseg] = j - i + 1;
+      segS[a.nseg] = f.istr[order[j]];
+      a.bx[a.nseg] = 1;
+      ++a.nseg;
+      i = j + 1;
+    }
+    for (int g = 0; g < a.nseg; ++g)
+      if (segS[g] & 1) return false;
+    return (f.istr[la] & 1) == 0;
+  };
+  auto divisor = [](int64_t d, int most) {   // the largest power of two dividing d, at most `most`
+    int b = 1;
+    while (b * 2 <= most && d % (b * 2) == 0) b *= 2;
+    return b;
+  };
+  auto inner = [&](int g) {   // index of run g's innermost axis
+    int ax = 0;
+    for (int q = 0; q < g; ++q) ax += a.seg_n[q];
+    return ax;
+  };
+  a.BZ = a.BY = 1;
+  a.y_outer = 0;
+  a.ostr_z = a.ostr_y = 0;
+  // Boxes of 8 KB or more.  Where la fills one tile of 16 or 32, an output run is 128 or 256
+  // bytes; the output axis next to it, ly, then becomes a run of its own and is boxed 4 (or 2)
+  // deep, and the run that is innermost in the input lengthens the reads.  2^27 elements, GB/s:
+  // seven axes reversed, la = 16: 5020 with 8 values of run 0 instead, 6090 with 4 of ly and 2 of
+  // the last run, 6040 with 2 and 4, 5170 with 8 and 1; la = 32: 4890, and 5940 with 2 and 2 (4
+  // and 1: 5670).  Otherwise the box takes several values of run 0's innermost axis.
+  int rz = -1, ry = -1;
+  const int ly = Da == TA && TA < 64 && la >= 1 && la - 1 != lb && f.dim[la - 1] % 2 == 0 ? la - 1 : -1;
+  if (ly >= 0 && cut_runs(ly, &ry)) {
+    rz = a.nseg - 1 == ry ? a.nseg - 2 : a.nseg - 1;   // the last run, other than ly's
+    a.BY = divisor(a.ax_dim[inner(ry)], TA == 16 ? 4 : 2);
+    a.ostr_y = a.ax_ostr[inner(ry)];
+    a.bx[ry] = a.BY;
+    if (rz >= 0) a.BZ = divisor(a.ax_dim[inner(rz)], 2);
+  } else {
+    if (!cut_runs(-1, &ry)) return false;
+    if (a.nseg > 0) {
+      rz = 0;
+      a.BZ = divisor(a.ax_dim[0], TA == 16 ? 8 : 64 / TA);
+    }
   }
+  if (rz >= 0) {
+    a.ostr_z = a.ax_ostr[inner(rz)];
+    a.bx[rz] = a.BZ;
+  }
+  a.y_outer = ry > rz;
   a.nbatch = 1;
-  for (int g = 1; g < a.nseg; ++g) a.nbatch *= a.segE[g];
-  if (a.nseg > 0) a.nbatch *= a.segE[0] / a.BZ;
+  for (int g = 0; g < a.nseg; ++g) a.nbatch *= a.segE[g] / a.bx[g];
   a.total = a.tiles_a * a.tiles_b * a.nbatch;
   a.wait_ns = kPermWaitNs;
   a.withhold = 0;
@@ -383,7 +424,8 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
     dims[2 + g] = (cuuint64_t)a.segE[g];
     strides[1 + g] = (cuuint64_t)segS[g] * 8;
   }
-  const cuuint32_t box[5] = {16, (cuuint32_t)TA, (cuuint32_t)a.BZ, 1, 1};
+  cuuint32_t box[5] = {16, (cuuint32_t)TA, 1, 1, 1};
+  for (int g = 0; g < a.nseg; ++g) box[2 + g] = (cuuint32_t)a.bx[g];
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, const_cast<void*>(in), dims, strides, box, estr,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -396,7 +438,7 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
 
 template <int TA, int NB>
 int launch_perm_tma(const PermTma& a, const CUtensorMap& map, float2* out, cudaStream_t st) {
-  const size_t smem = (size_t)NB * 16 * TA * 8 * a.BZ + 1024;   // NB x 8 or 16 KB
+  const size_t smem = (size_t)NB * 16 * TA * 8 * a.BZ * a.BY + 1024;   // NB x at most 16 KB
   static int attr_dev[64] = {0};
   int dev0 = 0;
   cudaGetDevice(&dev0);

@@ -317,6 +317,21 @@ def test_contract_step_odd_columns(qfx, variant, shape):
     assert np.all(np.abs(got - want) <= np.sqrt(2.0) * (2 * K + 1) * 2.0 ** -24 * scale)
 
 
+@pytest.mark.parametrize("case", [((16, 8, 3, 16), (3, 2, 1, 0)), ((16, 6, 5, 40), (3, 2, 1, 0)),
+                                  ((16, 4, 24), (2, 1, 0)), ((32, 2, 7, 18), (3, 2, 1, 0)),
+                                  ((2, 16, 3, 4, 32), (4, 2, 0, 3, 1)), ((4, 2, 32, 5, 16), (3, 4, 1, 0, 2)),
+                                  ((16, 3, 4, 33), (3, 1, 2, 0)), ((3, 8, 16, 2, 20), (4, 0, 3, 1, 2))])
+def test_permute_short_output_runs(qfx, case):
+    """Tensor-map transposes whose innermost output axis has 16 or 32 elements: the output axis
+    next to it is boxed too, where its extent has a factor 2, whatever its place in the input
+    (outermost, innermost or between), alone or beside a run that lengthens the reads."""
+    shape, perm = case
+    x = ri.random_complex(int(np.prod(shape)), seed=7)
+    out = qfx.permute(torch.from_numpy(x).cuda(), shape, perm)
+    qfx.sync()
+    np.testing.assert_array_equal(out.cpu().numpy(), primitives.permute(x, shape, perm).reshape(-1))
+
+
 @pytest.mark.parametrize("case", [((4, 5, 6), (2, 0, 1)), ((33, 65), (1, 0)),
                                   ((2, 3, 4, 5, 6), (4, 2, 0, 3, 1)), ((7, 8, 9), (0, 2, 1)),
                                   ((64, 3, 64), (2, 1, 0)), ((5, 1, 7), (1, 2, 0)),
