@@ -432,7 +432,8 @@ extern "C" qfx_status qfx_contract_step(const void* S, const void* B, void* C, i
   if (variant == 99 && tc) { flags = kTcWithhold; variant = -1; }
   if (variant == 12 && tc) { flags = kTcFast; variant = -1; }
   if (variant == 13 && tc) { flags = kTcNoTma; variant = -1; }
-  if (variant >= 0 && !simt_variant_valid(variant, 2))
+  // 24 and 29 (8 x 128 outputs) are the library's own choice only
+  if (variant == 24 || variant == 29 || (variant >= 0 && !simt_variant_valid(variant, 2)))
     return fail(QFX_EINVAL, "qfx_contract_step: unknown variant");
   if (variant >= 0 && !simt_variant_valid(variant, Sd))
     return fail(QFX_EINVAL, "qfx_contract_step: variants 0-4 and 20-23 need an even Sd");

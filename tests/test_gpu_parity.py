@@ -317,6 +317,24 @@ def test_contract_step_odd_columns(qfx, variant, shape):
     assert np.all(np.abs(got - want) <= np.sqrt(2.0) * (2 * K + 1) * 2.0 ** -24 * scale)
 
 
+@pytest.mark.parametrize("shape", [(1, 3, 8, 8, 126), (1, 64, 8, 4, 128), (65, 7, 5, 5, 2), (19, 33, 17, 17, 30),
+                                   (19456, 9, 8, 8, 2), (19, 33, 17, 17, 27), (129, 16, 8, 2, 1), (43, 8, 1, 1, 3)])
+def test_smallest_fill_tile(qfx, shape):
+    """Steps of a few rows on grids below one CTA per SM take the 8 x 128 tile (the library's own
+    choice; 19456 x 2 columns are its last grid on 152 SMs): partial tiles of rows and columns,
+    even and odd Sd.  The order of an output's sum is every tile's, so the bits are too."""
+    P, K, N, NL, Sd = shape
+    S = torch.from_numpy(ri.random_complex(K * N, seed=4)).cuda()
+    B = torch.from_numpy(ri.random_complex(P * K * Sd, seed=5)).cuda()
+    auto = qfx.contract_step(S, B, P, K, N, NL, Sd).cpu().numpy()
+    for v in (9, 28) + ((4, 23) if Sd % 2 == 0 else ()):
+        np.testing.assert_array_equal(auto, qfx.contract_step(S, B, P, K, N, NL, Sd, variant=v).cpu().numpy())
+    for v in (24, 29):
+        with pytest.raises(Exception, match="unknown variant"):
+            qfx.contract_step(S, B, P, K, N, NL, Sd, variant=v)
+    qfx.sync()
+
+
 @pytest.mark.parametrize("case", [((16, 8, 3, 16), (3, 2, 1, 0)), ((16, 6, 5, 40), (3, 2, 1, 0)),
                                   ((16, 4, 24), (2, 1, 0)), ((32, 2, 7, 18), (3, 2, 1, 0)),
                                   ((2, 16, 3, 4, 32), (4, 2, 0, 3, 1)), ((4, 2, 32, 5, 16), (3, 4, 1, 0, 2)),
