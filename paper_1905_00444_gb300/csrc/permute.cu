@@ -183,6 +183,7 @@ struct PermTma {
   int64_t ostr_b;           // output stride of lb
   int nseg;                 // runs of the other axes, contiguous in the input (<= 3)
   int64_t segE[3];          // run extents (coordinates 2..4 of the tensor map)
+  int64_t segT[3];          // and in boxes
   int seg_n[3];             // axes per run, innermost first
   int64_t ax_dim[kMaxRank], ax_ostr[kMaxRank];   // the runs' axes, run by run
   int bx[3];                // box extent along each run (divides its innermost axis)
@@ -202,27 +203,42 @@ struct TileMeta {
   int na, nb;
 };
 
+// x / d and x % d, in 32 bits where they hold it: a 64-bit division takes over a hundred clocks,
+// and the lane that issues the copies needs one per axis and tile
+__device__ __forceinline__ void perm_divmod(int64_t x, int64_t d, int64_t& q, int64_t& r) {
+  if (((uint64_t)x | (uint64_t)d) >> 32) {
+    const int64_t y = x / d;
+    r = x - y * d;
+    q = y;
+  } else {
+    const uint32_t x32 = (uint32_t)x, y = x32 / (uint32_t)d;
+    r = x32 - y * (uint32_t)d;
+    q = y;
+  }
+}
+
 // Thread 0: tensor-map coordinates and output placement of tile t; issues its copy.
 template <int TA>
 __device__ __forceinline__ void perm_issue(const PermTma& a, const CUtensorMap* map, int64_t t, uint32_t dst,
                                            uint32_t bar, TileMeta* meta) {
   constexpr int TB = 16;
-  const int64_t ta = t % a.tiles_a, r = t / a.tiles_a;
-  const int64_t tb = r % a.tiles_b;
-  int64_t bi = r / a.tiles_b;
+  int64_t ta, tb, bi, r;
+  perm_divmod(t, a.tiles_a, r, ta);
+  perm_divmod(r, a.tiles_b, bi, tb);
   int z[3] = {0, 0, 0};
   int64_t obase = ta * TA + tb * TB * a.ostr_b;
-  for (int g = a.nseg - 1; g >= 0; --g) {   // run 0 most significant; each advances a box at a time
-    const int64_t E = a.segE[g] / a.bx[g], zg = bi % E;
-    bi /= E;
+  for (int g = a.nseg - 1; g >= 1; --g) {   // run 0 most significant; each advances a box at a time
+    int64_t zg;
+    perm_divmod(bi, a.segT[g], bi, zg);
     z[g] = (int)(zg * a.bx[g]);
   }
+  if (a.nseg > 0) z[0] = (int)(bi * a.bx[0]);
   int ax = 0;
   for (int g = 0; g < a.nseg; ++g) {
     int64_t zg = z[g];
     for (int i = 0; i < a.seg_n[g]; ++i, ++ax) {
-      const int64_t c = zg % a.ax_dim[ax];
-      zg /= a.ax_dim[ax];
+      int64_t c = zg;
+      if (i + 1 < a.seg_n[g]) perm_divmod(zg, a.ax_dim[ax], zg, c);   // a run's last axis takes the rest
       obase += c * a.ax_ostr[ax];
     }
   }
@@ -237,12 +253,14 @@ __device__ __forceinline__ void perm_issue(const PermTma& a, const CUtensorMap* 
 // Warps 0-3 consume tiles; lane 0 of warp 4 issues the copies NB tiles ahead, reusing a
 // buffer once its 128 consumers have released it.  Every wait is bounded; a timeout sets
 // the status word and makes the other roles give up too.
-template <int TA, int NB>
+// Y: boxes along ly too (its index arithmetic costs other shapes up to a quarter)
+template <int TA, int NB, bool Y>
 __global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float2* __restrict__ out,
                                                           const __grid_constant__ CUtensorMap map) {
   constexpr int TB = 16;
-  const int TILE = TB * TA * 8 * a.BZ * a.BY, UNITS = 8 * (TA / 16) * a.BZ * a.BY;
-  const int by_shift = 31 - __clz(a.BY);   // BY is a power of two
+  const int BY = Y ? a.BY : 1;
+  const int TILE = TB * TA * 8 * a.BZ * BY, UNITS = 8 * (TA / 16) * a.BZ * BY;
+  const int by_shift = Y ? 31 - __clz(BY) : 0;   // BY is a power of two
   extern __shared__ char smem_raw[];
   // 128-byte swizzled boxes must start on 1024-byte boundaries
   char* buf = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -303,13 +321,14 @@ __global__ void __launch_bounds__(160) permute_tma_kernel(const PermTma a, float
     const char* tile = buf + b * TILE;
     for (int u = warp; u < UNITS; u += 4) {
       // iy fastest: neighbouring warps write neighbouring lines of an output run
-      const int iy = u & (a.BY - 1), w = u >> by_shift, c = w & 7;
+      const int iy = Y ? u & (BY - 1) : 0, w = Y ? u >> by_shift : u, c = w & 7;
       const int iz = (w >> 3) / (TA / 16), ia = ((w >> 3) % (TA / 16)) * 16 + ia_lo, ib = 2 * c + h;
-      const int row = (a.y_outer ? iy * a.BZ + iz : iz * a.BY + iy) * TA + ia;
+      const int row = (!Y ? iz : a.y_outer ? iy * a.BZ + iz : iz * BY + iy) * TA + ia;
       // a row of the box is 128 bytes of lb; its 16-byte chunk c sits at c ^ (row mod 8), and
       // row mod 8 = ia mod 8 since TA is a multiple of 8
       const float2 v = *reinterpret_cast<const float2*>(tile + row * 128 + ((c ^ (ia & 7)) << 4) + h * 8);
-      if (ia < m.na && ib < m.nb) out[m.obase + iy * a.ostr_y + iz * a.ostr_z + ia + (int64_t)ib * a.ostr_b] = v;
+      if (ia < m.na && ib < m.nb)
+        out[m.obase + (Y ? iy * a.ostr_y : 0) + iz * a.ostr_z + ia + (int64_t)ib * a.ostr_b] = v;
     }
     // the next copy into this buffer goes through the async proxy: order the reads first
     fence_async_smem();
@@ -386,7 +405,8 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   a.ostr_z = a.ostr_y = 0;
   // Boxes of 8 KB or more.  Where la fills one tile of 16 or 32, an output run is 128 or 256
   // bytes; the output axis next to it, ly, then becomes a run of its own and is boxed 4 (or 2)
-  // deep, and the run that is innermost in the input lengthens the reads.  2^27 elements, GB/s:
+  // deep, and the run that is innermost in the input lengthens the reads.  2^27 elements, GB/s, with
+  // four buffers a block (two give more, launch_perm_tma):
   // seven axes reversed, la = 16: 5020 with 8 values of run 0 instead, 6090 with 4 of ly and 2 of
   // the last run, 6040 with 2 and 4, 5170 with 8 and 1; la = 32: 4890, and 5940 with 2 and 2 (4
   // and 1: 5670).  Otherwise the box takes several values of run 0's innermost axis.
@@ -411,7 +431,10 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   }
   a.y_outer = ry > rz;
   a.nbatch = 1;
-  for (int g = 0; g < a.nseg; ++g) a.nbatch *= a.segE[g] / a.bx[g];
+  for (int g = 0; g < a.nseg; ++g) {
+    a.segT[g] = a.segE[g] / a.bx[g];
+    a.nbatch *= a.segT[g];
+  }
   a.total = a.tiles_a * a.tiles_b * a.nbatch;
   a.wait_ns = kPermWaitNs;
   a.withhold = 0;
@@ -436,27 +459,38 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   return true;
 }
 
-template <int TA, int NB>
+template <int TA, int NB, bool Y>
 int launch_perm_tma(const PermTma& a, const CUtensorMap& map, float2* out, cudaStream_t st) {
   const size_t smem = (size_t)NB * 16 * TA * 8 * a.BZ * a.BY + 1024;   // NB x at most 16 KB
   static int attr_dev[64] = {0};
   int dev0 = 0;
   cudaGetDevice(&dev0);
   if (dev0 < 64 && !attr_dev[dev0]) {
-    cudaError_t e = cudaFuncSetAttribute(permute_tma_kernel<TA, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(permute_tma_kernel<TA, NB, Y>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          NB * 16384 + 1024);   // boxes are at most 16 KB
     if (e != cudaSuccess) return (int)e;
     attr_dev[dev0] = 1;
   }
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // as many blocks per SM as 220 KB of shared memory holds, at most 8
-  int per_sm = (int)((220u << 10) / (smem + 512));
-  per_sm = per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm;
+  int sms = 0, l2 = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev0);
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev0);
+  // Blocks per SM, with two buffers each: tensors beyond L2 take four.  More copies in flight
+  // crowd the stores, fewer leave the memory idle.  2^27 elements (2^28 for the square), GB/s with
+  // 3 / 4 / 6 / 8 blocks, then 4 buffers and as many blocks as fit: seven axes reversed 5560 /
+  // 6300 / 5370 / 5370, 5550; 16384 x 16384 5930 / 6590 / 5180 / 5110, 5020; (16, 4096, 16, 128)
+  // reversed 5920 / 6200 / 5260 / 5250, 5350.  Tiles cut off at the edge of la or lb copy less
+  // and take more blocks for the same bytes: (64, 2, 89, 69, 32), half of whose tiles are 5 of 64
+  // wide, 3070 / 3670 / 4180 / 4530, 4620.  What L2 holds, or nearly, is bound by latency and
+  // takes eight; us with 4 / 6 / 8: (512, 106, 128) 22.6 / 19.9 / 18.5, 8192 x 1024 (134 MB in
+  // and out) 26.6 / 23.7 / 22.6; but 4096 x 4096 (268 MB) 46.9 / 51.9 / 53.4.  220 KB of shared
+  // memory are the limit, which six blocks of 16 KB boxes fill.
+  const int64_t tile_el = a.tiles_a * a.tiles_b * TA * 16, real_el = a.Da * a.Db;
+  const bool in_l2 = 16 * real_el * a.nbatch * a.BZ * a.BY <= (int64_t)l2 * 3 / 2;
+  int64_t per_sm = in_l2 ? 8 : std::min((4 * tile_el + real_el - 1) / real_el, (int64_t)8);
+  per_sm = std::min(per_sm, (int64_t)((220u << 10) / (smem + 512)));
   const int64_t want = (int64_t)(sms > 0 ? sms : 1) * per_sm;
   const unsigned grid = (unsigned)(a.total < want ? a.total : want);
-  permute_tma_kernel<TA, NB><<<grid, 160, smem, st>>>(a, out, map);
+  permute_tma_kernel<TA, NB, Y><<<grid, 160, smem, st>>>(a, out, map);
   return (int)cudaGetLastError();
 }
 }  // namespace
@@ -518,9 +552,12 @@ int launch_permute(const void* in, void* out, int rank, const int64_t* shape,
         tp.wait_ns = g_perm_withhold_ns;
         g_perm_withhold_ns = 0;
       }
-      const int err = TA == 64 ? launch_perm_tma<64, 4>(tp, map, dst, st)
-                    : TA == 32 ? launch_perm_tma<32, 4>(tp, map, dst, st)
-                               : launch_perm_tma<16, 4>(tp, map, dst, st);
+      const bool y = tp.BY > 1;
+      const int err = TA == 64 ? launch_perm_tma<64, 2, false>(tp, map, dst, st)
+                    : TA == 32 ? (y ? launch_perm_tma<32, 2, true>(tp, map, dst, st)
+                                    : launch_perm_tma<32, 2, false>(tp, map, dst, st))
+                               : (y ? launch_perm_tma<16, 2, true>(tp, map, dst, st)
+                                    : launch_perm_tma<16, 2, false>(tp, map, dst, st));
       count_launch();
       return err;
     }
