@@ -561,14 +561,13 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
               if (++nl == NL) { nl = 0; dst += strideNH - (int64_t)NL * a.Sd; }
             }
           } else {   // a chunk of a long contraction: add into C
-            // all 16 reads first (C is written only by this tile in this launch, so the
-            // read-only path applies): one memory latency per chunk, not one per element
+            // all 16 reads first: one memory latency per chunk, not one per element
             float2 o[16];
             float2* d = dst;
             int l = nl;
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              o[i] = __ldg(d);
+              o[i] = *d;
               d += a.Sd;
               if (++l == NL) { l = 0; d += strideNH - (int64_t)NL * a.Sd; }
             }
@@ -797,7 +796,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
         in.step(nbuf);
       }
     } else {
-      // rows that no tensor map describes: loads issued one k-stage ahead into registers
+      // rows that no tensor map describes: loads issued one k-stage ahead into registers (plain
+      // ones: the kernel that writes B may still run when this one starts)
       float2 nxt[SUB][KH];
       int64_t t = pair0;
       int it = 0;
@@ -816,7 +816,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
         for (int u = 0; u < SUB; ++u)
 #pragma unroll
           for (int kk = 0; kk < KH; ++kk)
-            nxt[u][kk] = inside && it * SUB + u < k_steps ? __ldg(src + (u * KS + kk) * a.Sd) : make_float2(0.f, 0.f);
+            nxt[u][kk] = inside && it * SUB + u < k_steps ? src[(u * KS + kk) * a.Sd] : make_float2(0.f, 0.f);
         src += SUB * KS * a.Sd;
         if (++it == KT) { it = 0; t += pairs; }
       };
@@ -1002,14 +1002,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
           int left = (nh0 + 1) * NL - n0;   // columns to the end of this nh
           float2* dst = Cj + nh0 * wrap + (int64_t)n0 * a.Sd;
           if (a.beta) {   // a chunk of a long contraction: add into C
-            // all 8 reads first (C is written only by this tile in this launch, so the
-            // read-only path applies): one memory latency per chunk, not one per element
+            // all 8 reads first: one memory latency per chunk, not one per element.  Plain
+            // loads: the launch of the chunk before may still be writing C while this one
+            // starts, and the read-only path is for memory that nothing writes meanwhile
             float2 o[8];
             const float2* d = dst;
             int l = left;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              o[e] = __ldg(d);
+              o[e] = *d;
               d += a.Sd;
               if (--l == 0) { l = NL; d += wrap; }
             }
