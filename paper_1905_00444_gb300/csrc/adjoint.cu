@@ -413,7 +413,7 @@ __host__ __device__ __forceinline__ int ev_slots(int kind) { return kind == EV_B
 
 __global__ void __launch_bounds__(kT) fold_backward_kernel(
     const FoldSite* __restrict__ sites, const FoldEvent* __restrict__ events, const float* __restrict__ matsf,
-    const CutDev* __restrict__ cuts, int n_cuts, const uint64_t* __restrict__ x1w, int64_t sid,
+    const CutDev* __restrict__ cuts, int n_cuts, const uint64_t* x1w, int64_t sid,
     const float2* sgrad, double* bpart, const int64_t* __restrict__ part_off) {
   launch_next();
   launch_wait();

@@ -33,7 +33,7 @@ template <int G>
 __global__ void __launch_bounds__(kThreads) fold_kernel(
     const FoldSite* __restrict__ sites, const FoldEvent* __restrict__ events,
     const float* __restrict__ matsf, const CutDev* __restrict__ cuts, int n_cuts,
-    const uint64_t* __restrict__ x1, int x1_words, int64_t n_batch, int64_t slice_begin,
+    const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
     int64_t item0, char* hdr, uint64_t hdr_stride, char* items, uint64_t item_bytes,
     uint64_t sites_off, int n_sites) {
   launch_next();
@@ -80,7 +80,7 @@ constexpr int kSmallSite = 1024;
 __global__ void __launch_bounds__(kSmallSite) fold_scale_kernel(
     const FoldSite* __restrict__ sites, const FoldEvent* __restrict__ events,
     const float* __restrict__ matsf, const CutDev* __restrict__ cuts, int n_cuts,
-    const uint64_t* __restrict__ x1, int x1_words, int64_t n_batch, int64_t slice_begin,
+    const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
     int64_t item0, char* hdr, uint64_t hdr_stride, char* items, uint64_t item_bytes,
     uint64_t sites_off, int n_sites) {
   launch_next();

@@ -64,7 +64,7 @@ __device__ __forceinline__ int64_t take_bits(int64_t& r, int32_t dim) {   // r m
   return v;
 }
 __device__ __forceinline__ FoldCoord fold_coord(const FoldSite& st, const CutDev* __restrict__ cuts, int n_cuts,
-                                                const uint64_t* __restrict__ x1w, int64_t sid, int64_t i) {
+                                                const uint64_t* x1w, int64_t sid, int64_t i) {
   int64_t off[4] = {0, 0, 0, 0};
   for (int c = 0; c < n_cuts; ++c) {
     const CutDev cd = cuts[c];
@@ -154,7 +154,7 @@ struct FoldState {
   cff v0[G], v1[G];
   bool split;
   __device__ __forceinline__ void begin(const FoldSite& st, const CutDev* __restrict__ cuts, int n_cuts,
-                                        const uint64_t* __restrict__ x1w, int64_t sid, int64_t i0) {
+                                        const uint64_t* x1w, int64_t sid, int64_t i0) {
 #pragma unroll
     for (int q = 0; q < G; ++q) fc[q] = fold_coord(st, cuts, n_cuts, x1w, sid, i0 + q);
     v0[0] = cff_one();

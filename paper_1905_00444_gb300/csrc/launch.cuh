@@ -4,8 +4,9 @@
 // are visible; a kernel that lets its successor start early says so once its own blocks are
 // running.  Between the small kernels of a sweep this hides most of the launch latency (all
 // amplitudes of 4x4x(1+16+1), 21 calls: 155 -> 122 us).
-// Such a kernel declares inputs that an earlier one writes without __restrict__: loads that the
-// compiler takes for invariant may move above the wait.
+// Such a kernel declares what an earlier one may write without __restrict__ and reads it with
+// plain loads: loads that the compiler takes for invariant may move above the wait.  The plan's
+// tables keep __restrict__: a copy ahead of a call's first kernel has written them.
 #pragma once
 
 #include <cuda_runtime.h>

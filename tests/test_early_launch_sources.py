@@ -43,3 +43,16 @@ def test_the_early_kernels_are_found():
 @pytest.mark.parametrize("kernel", early_kernels(), ids=lambda k: k[0])
 def test_no_read_only_loads(kernel):
     assert not re.search(r"__ldg|ld\.global\.(\w+\.)*nc", kernel[2])
+
+
+# the plan's tables, which a copy ahead of the call's first kernel has written
+TABLES = {"FoldSite": {"sites"}, "FoldEvent": {"events"}, "float": {"matsf"}, "CutDev": {"cuts"},
+          "int32_t": {"open_perm", "gate_ev"}, "int64_t": {"part_off"}}
+
+
+@pytest.mark.parametrize("kernel", early_kernels(), ids=lambda k: k[0])
+def test_restrict_is_for_tables_only(kernel):
+    for param in kernel[1].split(","):
+        if "__restrict__" in param:
+            kind, name = re.fullmatch(r"\s*const\s+(\w+)\s*\*\s*__restrict__\s+(\w+)\s*", param).groups()
+            assert name in TABLES.get(kind, ()), param
