@@ -183,6 +183,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   return true;
 }
+// Waits for work already in flight (copies, MMAs), whatever the abort flag says: after a timeout
+// it is still on its way, and neither TMEM nor the CTA may go before it has ended.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, unsigned long long limit_ns,
+                                           unsigned sleep_ns = 0) {
+  if (mbar_try(bar, parity)) return;
+  const unsigned long long deadline = globaltimer() + limit_ns;
+  while (!mbar_try(bar, parity) && globaltimer() < deadline)
+    if (sleep_ns) __nanosleep(sleep_ns);
+}
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   // K-major, no swizzle: LBO = 128 B (next core matrix along K), SBO = 256 B (next
   // 8-row group); bits 46-48 = 0b001; base offset 0; layout type 0.
@@ -465,10 +474,7 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       }
       // drain: every issued copy must land before the CTA exits
       for (int64_t i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i) {
-        const int s = (int)(i % STAGES);
-        const unsigned long long deadline = globaltimer() + kWaitNs;
-        while (!mbar_try(fullS(s), (uint32_t)((i / STAGES) & 1)) && globaltimer() < deadline) {
-        }
+        mbar_drain(fullS((int)(i % STAGES)), (uint32_t)((i / STAGES) & 1), kWaitNs);
       }
     }
   } else if (warp == 12) {
@@ -583,7 +589,7 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
     }
   }
 
-  if (warp == 12) mbar_wait(done, 0, abort, 256);   // last MMAs finished before freeing TMEM
+  if (warp == 12) mbar_drain(done, 0, kWaitNs, 256);   // last MMAs finished before freeing TMEM
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 12) {
@@ -686,6 +692,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   uint64_t* bars = reinterpret_cast<uint64_t*>(sIn + nbuf * CF::STAGE_IN);
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
+  __shared__ int site_pos, site_pass, site_issued;   // of the site stream at its end
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const int k_steps = (int)(a.K / KS);                // the last stage of a tile may have fewer
@@ -835,7 +842,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
     if (warp == 9 && lane == 0) {
       // ---- site image stream: per term the two planes of this CTA's half ---------------
       Ring st;
-      int64_t issued = 0;
+      int issued = 0;           // stages whose latest copy is this role's
       bool ok = !a.withhold_s;
       for (int64_t t = pair0; t < a.tiles && ok; t += pairs) {
         int64_t g, jt, nh;
@@ -854,22 +861,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
             src += (int64_t)a.NHt * (3 * TERMS) * planeS;
           }
           st.step(stages);
-          ++issued;
+          if (issued < stages) ++issued;
         }
       }
-      // every issued copy must land before the CTA exits: the MMAs that the leader waits for
-      // at the end read all of them, but after a timeout they may be in flight, so their
-      // barriers are watched here (a limit for each, as everywhere)
-      if (*abort) {
-        for (int64_t i = 0; i < (issued < stages ? issued : stages); ++i) {
-          st.i = st.i == 0 ? stages - 1 : st.i - 1;
-          if (st.i == stages - 1) st.pass ^= 1u;
-          const uint32_t bar = rank == 0 ? full(st.i) : fullS(st.i);
-          const unsigned long long deadline = globaltimer() + kWaitNs / 100;
-          while (!mbar_try(bar, st.pass) && globaltimer() < deadline) {
-          }
-        }
-      }
+      site_pos = st.i;
+      site_pass = (int)st.pass;
+      site_issued = issued;
     } else if (warp == 10 && lane == 0 && a.use_tma) {
       // ---- FP32 rows of B: one tensor-map copy per (tile, k-stage) into staging --------
       Ring in;
@@ -890,9 +887,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
       for (int64_t i = 0; i < (issued < nbuf ? issued : nbuf); ++i) {   // newest first
         in.i = in.i == 0 ? nbuf - 1 : in.i - 1;
         if (in.i == nbuf - 1) in.pass ^= 1u;
-        const unsigned long long deadline = globaltimer() + kWaitNs;
-        while (!mbar_try(in_full(in.i), in.pass) && globaltimer() < deadline) {
-        }
+        mbar_drain(in_full(in.i), in.pass, kWaitNs);
       }
     } else if (warp == 8 && lane == 0 && rank == 0) {
       // ---- MMA issue -------------------------------------------------------------------
@@ -1038,15 +1033,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   }
 
   __syncwarp();
-  if (warp == 8) mbar_wait(done, 0, abort, 256);   // last MMAs finished before freeing TMEM
+  if (warp == 8 && rank == 0) mbar_drain(done, 0, kWaitNs, 256);   // last MMAs finished before freeing TMEM
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  cluster_barrier();
+  cluster_barrier();   // the roles of both CTAs and all MMAs have ended
+  if (warp == 9 && lane == 0 && *abort) {
+    // after a timeout some site copies may have no MMA that waited for them
+    Ring st{site_pos, (uint32_t)site_pass};
+    for (int i = 0; i < site_issued; ++i) {   // newest first
+      st.i = st.i == 0 ? stages - 1 : st.i - 1;
+      if (st.i == stages - 1) st.pass ^= 1u;
+      mbar_drain(rank == 0 ? full(st.i) : fullS(st.i), st.pass, kWaitNs / 100);
+    }
+  }
   if (warp == 8) {
+    mbar_drain(done, 0, kWaitNs, 256);   // CTA 1: the last commit has arrived here as well
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
-  cluster_barrier();   // neither CTA leaves while the other still frees its half
+  cluster_barrier();   // neither CTA leaves while the other still frees its half or awaits an arrival
 }
 
 // Pre-split of the site matrix S[k][n] into the per-stage shared-memory image, per

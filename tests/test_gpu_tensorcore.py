@@ -249,3 +249,23 @@ def test_tensor_peak_probe(qfx):
     assert 0.35 < tf / bf < 0.65
     with pytest.raises(qfx.QfxError):
         qfx.tensor_peak("fp32")
+
+
+@pytest.mark.parametrize("prec,shape", [("bf16x3", (1, 256, 256, 256, 4096)), ("tf32x3", (3, 24, 64, 64, 30000)),
+                                        ("bf16x2", (700, 64, 128, 64, 130))])
+def test_bounded_wait_expires_on_many_pairs(qfx, prec, shape):
+    """The same on pairs with several tiles and stages (both CTAs give up, by tensor-map rows and
+    by per-thread loads), twice in a row; the next steps have the bits of the ones before."""
+    P, K, N, NL, Sd = shape
+    S = torch.from_numpy(ri.random_complex((K * N,), seed=1)).cuda()
+    B = torch.from_numpy(ri.random_complex((P * K * Sd,), seed=2)).cuda()
+    want = qfx.contract_step(S, B, P, K, N, NL, Sd, precision=prec)
+    qfx.sync()
+    for _ in range(2):
+        qfx.contract_step(S, B, P, K, N, NL, Sd, precision=prec, variant=99)
+        with pytest.raises(qfx.QfxError) as e:
+            qfx.sync()
+        assert e.value.status == qfx.qfx.QFX_ETIMEOUT
+        out = qfx.contract_step(S, B, P, K, N, NL, Sd, precision=prec)
+        qfx.sync()
+        assert torch.equal(out, want)
