@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(kSmallSite) fold_scale_kernel(
     f.run(sm, matsf, n);
   }
   float2 v = f.result(0);
-  const float mx = i < st.size ? fmaxf(fabsf(v.x), fabsf(v.y)) : 0.f;
+  // an entry that is no number counts as 0, as in fold_kernel: the others keep their scale
+  const float mx = i < st.size ? fmaxf(0.f, fmaxf(fabsf(v.x), fabsf(v.y))) : 0.f;
   const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
   __syncthreads();   // `largest` is cleared (also where a site has no events)
   if ((i & 31) == 0 && bits) atomicMax(&largest, bits);
