@@ -41,3 +41,23 @@ def test_scale_ignores_entries_that_overflow(qfx, items):
         if x & 0b1001 == 0:
             want = 1e-50 * psi[x]
             assert np.all(np.abs(got[:, j] - want) <= 1e-5 * max(abs(want), 1e-50 * 2.0 ** -2)), (j, got[0, j], want)
+
+
+@pytest.mark.parametrize("shape,n_batch", [((2, 2, 56), 160), ((1, 2, 64), 640)])
+def test_more_events_than_one_stage_holds(qfx, shape, n_batch):
+    """72 and 74 events a site, above the 64 that one stage in shared memory holds.  (2, 2, 56):
+    one item of 2^14-element sites takes an element per thread; (1, 2, 64): one item of 256
+    elements folds and scales in one launch; all items together take groups of four.  The same
+    bits, and the state vector's amplitudes."""
+    rows, cols, d = shape
+    c = ri.rqc(rows, cols, d, seed=5)
+    plan = qfx.Plan(qfx.Circuit(c), n_open=1)
+    x1s = ri.random_bitstrings(rows * cols, n_batch, seed=6)
+    many = amplitudes(qfx, plan, x1s, n_batch)
+    one = torch.cat([amplitudes(qfx, plan, x1s[i:i + 1], 1) for i in range(0, n_batch, 53)])
+    assert torch.equal(many[::53], one)
+    psi = statevector.amplitudes(c)
+    q = plan.open_sites[0]
+    want = np.array([[psi[(int(x) & ~(1 << q)) | (j << q)] for j in range(2)] for x in x1s])
+    err = np.abs(many.cpu().numpy() - want)
+    assert np.all(err <= 1e-5 * np.maximum(np.abs(want), 2.0 ** (-rows * cols / 2)))
