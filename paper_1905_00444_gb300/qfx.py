@@ -6,6 +6,7 @@ fallback path.
 from __future__ import annotations
 
 import ctypes as C
+import operator
 import os
 import re
 from typing import Iterable, List, Optional, Sequence
@@ -149,6 +150,7 @@ def launch_count() -> int:
 GATE_DTYPE = np.dtype([("layer", np.int32), ("q0", np.int32), ("q1", np.int32), ("kind", np.int32),
                        ("mat", np.complex128, 16)])
 assert GATE_DTYPE.itemsize == C.sizeof(Gate)
+_FIELDS = operator.attrgetter("layer", "q0", "q1", "kind")
 
 
 def gate_table(gates, mats):
@@ -158,8 +160,13 @@ def gate_table(gates, mats):
     table = np.zeros(max(1, len(gates)), dtype=GATE_DTYPE)
     if not gates:
         return table
-    table["layer"], table["q0"], table["q1"], table["kind"] = zip(
-        *[(g.layer, g.q0, g.q1, g.kind) for g in gates])
+    for name, column in zip(("layer", "q0", "q1", "kind"), zip(*map(_FIELDS, gates))):
+        # what is not integers of 32 bits goes through the ABI's own type, which refuses or wraps it
+        try:
+            plain = all(issubclass(t, (int, np.integer)) for t in set(map(type, column)))
+            table[name] = column if plain else [C.c_int32(v).value for v in column]
+        except OverflowError:
+            table[name] = [C.c_int32(v).value for v in column]
     if isinstance(mats, np.ndarray):
         table["mat"][:, :mats.shape[1]] = mats
         return table
@@ -170,6 +177,15 @@ def gate_table(gates, mats):
         rows = np.flatnonzero(sizes == size)
         table["mat"][rows, :size] = np.array([mats[i] for i in rows])
     return table
+
+
+def _entries(mat):
+    """A gate matrix's entries in a row: a numpy array's, or those of any array-like object with
+    reshape whose scalars have .real and .imag (a torch tensor, on any device)."""
+    flat = mat.reshape(-1)
+    if isinstance(flat, np.ndarray):
+        return flat
+    return np.array([complex(float(v.real), float(v.imag)) for v in flat], dtype=np.complex128)
 
 
 def _stream_ptr(stream) -> Optional[int]:
@@ -192,8 +208,7 @@ class Circuit:
             self.n_gates = sum(1 for ln in text.splitlines()
                                if ln.split("#")[0].strip() and not ln.strip().startswith("grid"))
         else:
-            self._create(src.rows, src.cols, src.gates,
-                         [np.asarray(g.mat).reshape(-1) for g in src.gates], h)
+            self._create(src.rows, src.cols, src.gates, [_entries(g.mat) for g in src.gates], h)
         self._h = h
 
     def _create(self, rows, cols, gates, mats, h):
