@@ -4,6 +4,7 @@ adjoint contraction (qfx_amplitudes_backward); both run in the library's kernels
 from __future__ import annotations
 
 import copy
+import math
 from typing import Optional, Sequence
 
 from . import qfx
@@ -39,13 +40,17 @@ class _Rebuilt:
 
 
 def _circuit_with(template, gates_host):
-    """The template with its gate matrices replaced by the rows of gates_host."""
-    width = gates_host.shape[1]
-    if width < 4:
-        raise ValueError("gates rows need at least 4 entries")
-    if width != 16 and any(g.q1 >= 0 and g.mat.size == 16 for g in template.gates):
+    """The template with its gate matrices replaced by the rows of gates_host: [n, 4] or [n, 16]
+    entries, or rows of any shape ([n, 2, 2], ...) whose first 4 elements are 4 values, and whose
+    values are 16 where a gate is general."""
+    rows = gates_host.reshape(len(gates_host), math.prod(gates_host.shape[1:]))
+    first = math.prod(gates_host[:1, :4].shape[1:])
+    general = [g.q1 >= 0 and g.mat.size == 16 for g in template.gates[:len(rows)]]
+    if any(general) and rows.shape[1] != 16:
         raise ValueError("a general (U4) gate needs gates rows of 16 entries")
-    return _Rebuilt(template, gates_host[:, :16])
+    if first != 4 and not all(general):
+        raise ValueError("gates rows need at least 4 entries")
+    return _Rebuilt(template, rows[:, :16 if any(general) else 4])
 
 
 def _make():
