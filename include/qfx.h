@@ -338,8 +338,9 @@ uint64_t qfx_backward_workspace_bytes(const qfx_plan* p);
 
 /* Autotuner: times every compatible FP32 tile variant of each distinct step shape of `p`
  * (on `workspace`, shrinking the problem to fit it) and records the fastest per shape
- * (N, K, NL, Sd) in the JSON file `cache_path` (existing entries are kept and not
- * re-timed).  Plans created with opts.autotune_cache use the recorded variants.
+ * (N, K, NL, Sd) in the JSON file `cache_path` (existing entries of the present tiles are
+ * kept and not re-timed; those timed on an earlier version's tiles are dropped).  Plans created
+ * with opts.autotune_cache use the recorded variants, and ignore those of other tiles.
  * Synchronises `stream`.  Errors: QFX_EINVAL, QFX_ENOMEM, QFX_ECUDA. */
 qfx_status qfx_autotune(const qfx_plan* p, const char* cache_path, void* workspace,
                         size_t ws_bytes, void* stream);

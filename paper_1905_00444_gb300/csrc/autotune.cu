@@ -5,9 +5,12 @@
 // precision and its tensor-core flags.  qfx_plan_create with qfx_plan_opts.autotune_cache
 // applies the cached choices; shapes not in the cache keep the planner's default.  Format:
 //   {"qfx_autotune": 1, "entries": [
-//     {"N": 256, "K": 256, "NL": 256, "Sd": 1048576, "prec": 0, "tc_flags": 0,
-//      "variant": 0, "ms": 1.23}, ...]}
+//     {"N": 256, "K": 256, "NL": 256, "Sd": 1048576, "prec": 0, "tc_flags": 0, "tiles": 2,
+//      "variant": 1, "ms": 1.23}, ...]}
 // A variant of 10 or more stands for the tensor-core kernel of the entry's precision.
+// "tiles" says which set of tiles the entry was timed on.  What another set has timed (the first
+// one wrote "prec" and no "tiles") is ignored, and timed again: its variants name other tiles.  An
+// entry with neither is a user's own choice and holds for any set.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,6 +26,10 @@
 
 namespace qfx {
 namespace {
+
+// The tiles behind the variants 0-9 and the tensor-core kernels; to be counted up with them, so that
+// times of other tiles are not taken for theirs.
+constexpr int kTileSet = 2;
 
 using Key = std::tuple<int64_t, int64_t, int64_t, int64_t, int, int>;   // N, K, NL, Sd, prec, tc flags
 struct Entry {
@@ -65,8 +72,14 @@ std::map<Key, Entry> read_cache(const char* path) {
     if (number_after(e, "N", &N) && number_after(e, "K", &K) && number_after(e, "NL", &NL) &&
         number_after(e, "Sd", &Sd) && number_after(e, "variant", &v)) {
       number_after(e, "ms", &ms);
-      number_after(e, "prec", &prec);
+      const bool timed = number_after(e, "prec", &prec);
       number_after(e, "tc_flags", &fl);
+      double tiles = timed ? 1 : kTileSet;
+      number_after(e, "tiles", &tiles);
+      if (tiles != kTileSet) {
+        pos = b + 1;
+        continue;
+      }
       if (v >= 0 && (v < 10 || (prec > 0 && v == kVariantTcBf16)))
         out[Key{(int64_t)N, (int64_t)K, (int64_t)NL, (int64_t)Sd, (int)prec, (int)fl}] = Entry{(int)v, ms};
     }
@@ -84,6 +97,7 @@ bool write_cache(const char* path, const std::map<Key, Entry>& m) {
     f << "  {\"N\": " << std::get<0>(kv.first) << ", \"K\": " << std::get<1>(kv.first)
       << ", \"NL\": " << std::get<2>(kv.first) << ", \"Sd\": " << std::get<3>(kv.first)
       << ", \"prec\": " << std::get<4>(kv.first) << ", \"tc_flags\": " << std::get<5>(kv.first)
+      << ", \"tiles\": " << kTileSet
       << ", \"variant\": " << kv.second.variant << ", \"ms\": " << kv.second.ms << "}"
       << (++i < m.size() ? ",\n" : "\n");
   }

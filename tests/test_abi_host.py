@@ -296,6 +296,28 @@ def test_autotune_cache_is_applied(tmp_path):
     assert [st["variant"] for st in p2.steps] == [st["variant"] for st in base.steps]
 
 
+@pytest.mark.parametrize("entry,applied", [('"prec": 0, "tc_flags": 0', False),
+                                           ('"prec": 0, "tc_flags": 0, "tiles": 1', False),
+                                           ('"prec": 0, "tc_flags": 0, "tiles": 3', False),
+                                           ('"prec": 0, "tc_flags": 0, "tiles": 2', True),
+                                           ('"tiles": 1', False), ('"tiles": 2', True)])
+def test_autotune_entries_of_other_tiles_are_ignored(tmp_path, entry, applied):
+    """What was timed on another set of tiles chooses nothing: its variants name other tiles."""
+    c = ri.rqc(4, 4, 16, seed=0)
+    base = qfx.Plan(qfx.Circuit(c), n_open=3)
+    s = next(st for st in base.steps[1:] if st["Sd"] % 2 == 0 and st["N"] >= 16)
+    other = 2 if s["variant"] != 2 else 1
+    cache = tmp_path / "tune.json"
+    cache.write_text('{"qfx_autotune": 1, "entries": [\n'
+                     f'  {{"N": {s["N"]}, "K": {s["K"]}, "NL": {s["NL"]}, "Sd": {s["Sd"]}, {entry}, '
+                     f'"variant": {other}, "ms": 0.5}}\n]}}\n')
+    tuned = qfx.Plan(qfx.Circuit(c), n_open=3, autotune_cache=str(cache))
+    if not applied:
+        assert tuned.steps == base.steps
+    else:
+        assert any(b["variant"] == other and a["variant"] != other for a, b in zip(base.steps, tuned.steps))
+
+
 def test_autograd_circuit_rows_of_sixteen_entries():
     """The autograd wrapper rebuilds the template from [n, 16] rows: 2x2 from the first 4
     of a single-qubit gate, the diagonal from the first 4 of a CZ, the 4x4 of a U4 gate;

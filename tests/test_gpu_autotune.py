@@ -60,3 +60,18 @@ def test_autotune_chooses_between_tensor_cores_and_fp32_tiles(qfx, tmp_path, pre
     got = qfx.amplitudes(tuned, x1).cpu().numpy()
     qfx.sync()
     assert np.linalg.norm(got - ref) <= 3e-5 * np.linalg.norm(ref)
+
+
+def test_entries_of_other_tiles_are_timed_again(qfx, tmp_path):
+    """A file from before the present tiles: every shape is timed again and its entry replaced."""
+    plan = qfx.Plan(qfx.Circuit(ri.rqc(4, 4, 16, seed=3)), n_open=5)
+    cache = tmp_path / "tune.json"
+    old = [{"N": s["N"], "K": s["K"], "NL": s["NL"], "Sd": s["Sd"], "prec": 0, "tc_flags": 0, "variant": 5,
+            "ms": 1e6} for s in plan.steps[1:]]
+    cache.write_text(json.dumps({"qfx_autotune": 1, "entries": old}))
+    qfx.autotune(plan, str(cache))
+    qfx.sync()
+    entries = json.loads(cache.read_text())["entries"]
+    key = lambda e: (e["N"], e["K"], e["NL"], e["Sd"])  # noqa: E731
+    assert {key(e) for e in entries} == {key(e) for e in old}
+    assert all(e["ms"] < 1e6 and e["tiles"] == 2 for e in entries)
