@@ -706,7 +706,7 @@ def measure_batch(qfx, torch, mix, n_open, steps, warmup, tc, autotune):
                                "items_per_s": len(items) / t_graph, "tasks_or_graph_nodes": n_tasks_fp32,
                                "slots": slots_fp32,
                                "what": "one batch replayed from a CUDA graph: items with steps of "
-                                       ">= 1024 tiles as their own launches, the others in one "
+                                       ">= 1024 tiles (512 of 8 rows) as their own launches, the others in one "
                                        "persistent launch"},
            "fp32_per_item": {"value": flops / t_items / 1e12, "ms_per_batch": 1e3 * t_items,
                              "items_per_s": len(items) / t_items, "kernel_launches": per_item_launches},

@@ -265,11 +265,11 @@ qfx_status qfx_amplitudes_static(const qfx_plan* p, const uint64_t* x1, int64_t 
  * Many work items -- every (slice, x1) of every listed item, of any mix of plans and
  * shapes -- run together:
  * - items whose steps all run FP32 tiles (FP32 plans, and split-precision plans whose
- *   step shapes the tensor-core tile does not take) and whose largest step has fewer
- *   than 1024 output tiles: in ONE persistent kernel, a device task queue of fold chunks,
- *   scale chunks, contraction-step tiles (each step's plan-chosen variant) and FP64
- *   accumulations, with per-segment completion counters as dependencies and bounded
- *   waits;
+ *   step shapes the tensor-core tile does not take) and whose steps all have fewer than
+ *   1024 output tiles (512 of those of 8 rows, N < 16): in ONE persistent kernel, a device
+ *   task queue of fold chunks, scale chunks, contraction-step tiles (each step's
+ *   plan-chosen variant) and FP64 accumulations, with per-segment completion counters as
+ *   dependencies and bounded waits;
  * - items with tensor-core steps, larger items and contraction trees: as ONE CUDA graph
  *   built at prepare time, every item's launch sequence on one of up to 16 parallel
  *   lanes, each lane with its own workspace slot (`slots` = lanes); the persistent

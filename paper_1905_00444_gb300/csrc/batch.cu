@@ -341,21 +341,24 @@ struct qfx_batch {
 
 using namespace qfx;
 
-// Whether an FP32 work item runs as its own launch sequence in a batch's graph: its
-// largest step has at least kBigTiles output tiles, so the step kernels fill the GPU many
-// times over and launch overhead is negligible, while the same tiles run slower inside the
-// persistent kernel (measured with tiles of twice the columns, 512 of which drew the line at
-// the same step sizes: 48.2 against 41.6 TFLOP/s on the mixed-grid batch).
-constexpr int64_t kBigTiles = 1024;
+// Whether an FP32 work item runs as its own launch sequence in a batch's graph: a step of its
+// plan has at least this many output tiles, so the step kernels fill the GPU many times over
+// and launch overhead is negligible, while the same tiles run slower inside the persistent
+// kernel, and so do the accumulations of many outputs (one task each).  16 items, 16 slots, ms in
+// the persistent kernel and as launches: 1024 tiles of 64 x 128 (6x6x24, 2^9 outputs) 10.2 and
+// 8.4; 2048 (7x7x24) 83.9 and 69.6; 512 tiles of 8 x 512 (4x5x8, 2^19 outputs) 3.36 and 0.79.
+// Below the line launches still gain at 256 tiles (6x6x24, 2^4 outputs: 7.5 and 6.3) and lose at
+// 64 (8x8x16: 1.46 and 1.65); it stands where it stood when the tiles of 16 to 64 rows had twice
+// the columns and those of 8 rows the same.
+int64_t big_tiles(int variant) { return variant % 5 == 4 ? 512 : 1024; }
 bool item_is_big(const qfx_plan* p) {
   if (p->family == 1) return true;   // contraction trees run through the launch path only
-  int64_t most = 0;
   for (size_t i = 1; i < p->steps.size(); ++i) {
     const Step& sp = p->steps[i];
     const int v = sp.variant >= kVariantTcBf16 ? pick_variant(sp.N, sp.Sd) : sp.variant;
-    most = std::max(most, step_tiles(v, sp.N, sp.P * sp.Sd));
+    if (step_tiles(v, sp.N, sp.P * sp.Sd) >= big_tiles(v)) return true;
   }
-  return most >= kBigTiles;
+  return false;
 }
 
 // Whether a work item runs as its own launch sequence in a batch's graph rather than inside
