@@ -15,18 +15,19 @@
 //
 // Tiles: the boundary tensor B is the A operand (rows j), the site matrix S the B operand
 // (rows n), pre-split once per step by split_site_kernel into the shared-memory image of its
-// term planes.  Default tiles (cgemm_pair_kernel) are 256 rows j by Nt <= 128 columns n on a
-// pair of CTAs, with split accumulators in TMEM: hi x hi products go to "main" accumulators,
-// every cross-term product to "small" ones, added in the epilogue, so that the large
-// accumulators see two additions per k-step.  There the complex product is embedded in N: S is
-// held per term as planes Sr, Si, -Sr, and one MMA of N = 2 Nt takes Ar x [Sr; Si] into
-// (re, im) and another -Ai x [Si; -Sr], so each MMA reads A once for both halves.
-// QFX_TC_FAST_ACCUMULATION tiles (cgemm_fast_kernel) are 128 x 256 on one CTA with one
-// accumulator pair (re [0,256), im [256,512)) and four real products per term pair (4M).
-// Both kernels are persistent: producer warps split FP32 rows of B into term planes (K-major,
+// term planes.  Default tiles are 256 rows j by Nt <= 128 columns n on a pair of CTAs
+// (cgemm_pair_kernel), or for short contractions 128 rows on one CTA (cgemm_cta_kernel), with
+// split accumulators in TMEM: hi x hi products go to "main" accumulators, every cross-term
+// product to "small" ones, added in the epilogue, so that the large accumulators see two
+// additions per k-step.  There the complex product is embedded in N: S is held per term as planes
+// Sr, Si, -Sr, and one MMA of N = 2 Nt takes Ar x [Sr; Si] into (re, im) and another
+// -Ai x [Si; -Sr], so each MMA reads A once for both halves.
+// QFX_TC_FAST_ACCUMULATION tiles (cgemm_cta_kernel too) are 128 x 256 with one accumulator pair
+// (re [0,256), im [256,512)) and four real products per term pair (4M).
+// The kernels are persistent: producer warps split FP32 rows of B into term planes (K-major,
 // no-swizzle core-matrix layout), one thread issues the MMAs, others stream the site image with
-// bulk copies and, for pairs, the rows of B with tensor-map copies into staging buffers when
-// the shape allows it, and epilogue warps drain TMEM into C.
+// bulk copies and, for default tiles, the rows of B with tensor-map copies into staging buffers
+// when the shape allows it, and epilogue warps drain TMEM into C.
 // Rings of shared-memory stages are guarded by mbarriers.  Every wait has a deadline;
 // on expiry the kernel records an error, drains its own copies and MMAs, frees TMEM and
 // returns (the host reports QFX_ETIMEOUT).
@@ -351,36 +352,46 @@ __device__ __forceinline__ void split_row(const TcArgs& a, int64_t j, int64_t& p
   }
 }
 
-// ---- fast accumulation: one CTA per SM, one accumulator pair -------------------------
-// re in TMEM columns [0, Nt), im in [256, 256 + Nt).  Warps: 0-3 producers, 4-11 epilogue (two
-// per TMEM lane quarter, each half the columns), 12 TMEM owner + MMA issuer, 13 site stream.
-template <int MODE>
-struct FastCfg {
+// ---- tiles on one CTA -------------------------------------------------------------------
+// 128 rows j on one CTA per SM.  SPLIT: default accumulation of steps of few k-steps
+// (takes_cta_tile), Nt <= 128, main accumulators in TMEM columns [0, 2 Nt), small ones in [256,
+// 256 + 2 Nt), each re then im.  Otherwise fast accumulation, Nt <= 256: re in [0, Nt), im in [256,
+// 256 + Nt).  Warps: 0-3 producers, 4-11 epilogue (two per TMEM lane quarter, each half the
+// columns), 12 TMEM owner + MMA issuer, 13 site stream and tensor-map copies.
+template <int MODE, bool SPLIT>
+struct CtaCfg {
   using M_ = Mode<MODE>;
-  static constexpr int NT_MAX = 256;
-  static constexpr int PLANES = 2 * M_::TERMS;             // planes of each operand per stage
-  static constexpr int STAGES = 3;
+  static constexpr int NT_MAX = SPLIT ? 128 : 256;
+  static constexpr int PLANES = 2 * M_::TERMS;             // planes of B per stage
+  static constexpr int SPLANES = SPLIT ? 3 * M_::TERMS : PLANES;   // and of S
+  static constexpr int STAGES = SPLIT ? (M_::TERMS == 3 ? 3 : 4) : 3;
   static constexpr int STAGE_A = PLANES * kPlaneA;
+  static constexpr int STAGE_IN = kRows * M_::KS * 8;
+  // staging buffers of tensor-map copies; the operand ring of the fast tile leaves no room for them
+  static constexpr int NBUF = SPLIT ? (M_::KS == 16 ? 2 : 4) : 0;
   static constexpr int THREADS = 14 * 32;
   static size_t smem(int nt) {
-    return kAlignPad + (size_t)STAGES * (STAGE_A + PLANES * nt * 32) + (3 * STAGES + 3) * sizeof(uint64_t);
+    return kAlignPad + (size_t)STAGES * (STAGE_A + SPLANES * nt * 32) + (size_t)NBUF * STAGE_IN +
+           (3 * STAGES + 3 + 2 * NBUF) * sizeof(uint64_t);
   }
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(const TcArgs a) {
+template <int MODE, bool SPLIT>
+__global__ void __launch_bounds__(CtaCfg<MODE, SPLIT>::THREADS, 1)
+    cgemm_cta_kernel(const TcArgs a, const __grid_constant__ CUtensorMap tmA) {
   using M_ = Mode<MODE>;
-  using CF = FastCfg<MODE>;
+  using CF = CtaCfg<MODE, SPLIT>;
   constexpr int TERMS = M_::TERMS, KS = M_::KS, STAGES = CF::STAGES;
   extern __shared__ __align__(16) char smem_raw[];
   char* smem = smem_raw + ((kAlignPad - (smem_u32(smem_raw) & (kAlignPad - 1))) & (kAlignPad - 1));
   const int stageA = CF::STAGE_A;
   const int planeS = a.Nt * 32;
-  const int stageS = CF::PLANES * planeS;
+  const int stageS = CF::SPLANES * planeS;
   char* sA = smem;
   char* sS = smem + STAGES * stageA;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sS + STAGES * stageS);
-  // bars: fullA[S], fullS[S], empty[S], acc_full, tmem_free, done
+  char* sIn = sS + STAGES * stageS;                 // NBUF x [box_p][KS][box_s] float2
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sIn + CF::NBUF * CF::STAGE_IN);
+  // bars: fullA[S], fullS[S], empty[S], acc_full, tmem_free, done, in_full[NBUF], in_empty[NBUF]
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -392,6 +403,8 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
   const uint32_t acc_full = smem_u32(&bars[3 * STAGES]);
   const uint32_t tmem_free = smem_u32(&bars[3 * STAGES + 1]);
   const uint32_t done = smem_u32(&bars[3 * STAGES + 2]);
+  auto in_full = [&](int b) { return smem_u32(&bars[3 * STAGES + 3 + b]); };
+  auto in_empty = [&](int b) { return smem_u32(&bars[3 * STAGES + 3 + CF::NBUF + b]); };
 
   if (tid == 0) {
     abort_flag = 0;
@@ -403,8 +416,15 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
     mbar_init(acc_full, 1);
     mbar_init(tmem_free, 8);
     mbar_init(done, 1);
+    for (int b = 0; b < CF::NBUF; ++b) {
+      mbar_init(in_full(b), 1);
+      mbar_init(in_empty(b), kRows);
+    }
     mbar_init_fence();
   }
+  launch_next();
+  launch_wait();       // the site image is written; before the TMEM, which an earlier kernel may hold
+  __syncwarp();
   if (warp == 12) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_base_slot))
                  : "memory");
@@ -418,14 +438,46 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
 
   if (warp < 4) {
     // ---- producers: split 128 rows of B per k-stage into term planes -------------------
-    // Rows are loaded one k-stage ahead into registers, so that their latency overlaps the
+    // Rows arrive through tensor-map copies staged NBUF k-stages ahead (issued by warp 13), or
+    // through loads issued one k-stage ahead into registers, so that their latency overlaps the
     // split and the wait for a free operand stage.
     int64_t t = blockIdx.x, it = 0, q = 0;
+    if (CF::NBUF > 0 && a.use_tma) {
+      constexpr int NB = CF::NBUF > 0 ? CF::NBUF : 1;
+      const int ps = tid / a.box_s, ss = tid % a.box_s;     // this row inside the box
+      while (t < a.tiles && !*abort) {
+        const int b = (int)(q % NB);
+        if (!mbar_wait(in_full(b), (uint32_t)((q / NB) & 1), abort)) break;
+        const float2* in = reinterpret_cast<const float2*>(sIn + b * CF::STAGE_IN);
+        float re[KS], im[KS];
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) {
+          const float2 v = in[(ps * KS + kk) * a.box_s + ss];
+          re[kk] = v.x;
+          im[kk] = v.y;
+        }
+        // the next tensor-map copy rewrites this buffer through the async proxy: order these
+        // generic reads before it
+        fence_async_smem();
+        mbar_arrive(in_empty(b));
+        const int s = (int)(q % STAGES);
+        if (q >= STAGES && !mbar_wait(empty(s), (uint32_t)((q / STAGES - 1) & 1), abort)) break;
+        char* st = sA + s * stageA;
+        store_row_terms<MODE>(st, kPlaneA, tid, re);
+        store_row_terms<MODE>(st + TERMS * kPlaneA, kPlaneA, tid, im);
+        fence_async_smem();
+        mbar_arrive(fullA(s));
+        ++q;
+        if (++it == KT) { it = 0; t += gridDim.x; }
+      }
+    } else {
     auto row_ptr = [&](int64_t tt, int64_t& pofs) -> const float2* {
       int64_t g, jt, nh;
       tile_coords(a, tt, g, jt, nh);
       const int64_t jg = jt * kRows + tid;
-      pofs = jg < a.J ? (jg / a.Sd) * a.K * a.Sd + (jg % a.Sd) : -1;
+      int64_t p, sidx;
+      split_row(a, jg, p, sidx);
+      pofs = jg < a.J ? p * a.K * a.Sd + sidx : -1;
       return a.B + g * a.b_stride;
     };
     float2 nxt[KS];
@@ -434,7 +486,7 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       const float2* Bg = row_ptr(tt, pofs);
 #pragma unroll
       for (int kk = 0; kk < KS; ++kk)
-        nxt[kk] = pofs >= 0 ? __ldg(Bg + pofs + (ii * KS + kk) * a.Sd) : make_float2(0.f, 0.f);
+        nxt[kk] = pofs >= 0 ? Bg[pofs + (ii * KS + kk) * a.Sd] : make_float2(0.f, 0.f);
     };
     if (t < a.tiles) fetch(t, 0);
     while (t < a.tiles && !*abort) {
@@ -454,6 +506,7 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       ++q;
       t = nt;
       it = ni;
+    }
     }
   } else if (warp == 13) {
     // ---- S image stream ------------------------------------------------------------
@@ -476,13 +529,32 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       for (int64_t i = (issued > STAGES ? issued - STAGES : 0); i < issued; ++i) {
         mbar_drain(fullS((int)(i % STAGES)), (uint32_t)((i / STAGES) & 1), kWaitNs);
       }
+    } else if (lane == 1 && CF::NBUF > 0 && a.use_tma) {
+      // ---- FP32 rows of B: one tensor-map copy per (tile, k-stage) into staging --------
+      constexpr int NB = CF::NBUF > 0 ? CF::NBUF : 1;
+      int64_t q = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+        int64_t g, jt, nh, p, sidx;
+        tile_coords(a, t, g, jt, nh);
+        split_row(a, jt * kRows, p, sidx);
+        for (int64_t it = 0; it < KT; ++it, ++q) {
+          const int b = (int)(q % NB);
+          if (q >= NB && !mbar_wait(in_empty(b), (uint32_t)((q / NB - 1) & 1), abort, 32)) { ok = false; break; }
+          mbar_arrive_tx(in_full(b), (uint32_t)CF::STAGE_IN);
+          tma_load_4d(smem_u32(sIn + b * CF::STAGE_IN), &tmA, (int)sidx, (int)(it * KS), (int)p, (int)g, in_full(b));
+        }
+      }
+      for (int64_t i = (q > NB ? q - NB : 0); i < q; ++i)
+        mbar_drain(in_full((int)(i % NB)), (uint32_t)((i / NB) & 1), kWaitNs);
     }
   } else if (warp == 12) {
     // ---- MMA issue -----------------------------------------------------------------
     if (lane == 0) {
       int64_t q = 0, tc = 0;
       bool ok = true;
-      const uint32_t idesc_p = instr_desc<MODE>(a.Nt, false), idesc_n = instr_desc<MODE>(a.Nt, true);
+      const int n_mma = SPLIT ? 2 * a.Nt : a.Nt;
+      const uint32_t idesc_p = instr_desc<MODE>(n_mma, false), idesc_n = instr_desc<MODE>(n_mma, true);
       for (int64_t t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tc) {
         if (tc > 0 && !mbar_wait(tmem_free, (uint32_t)((tc - 1) & 1), abort)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -493,7 +565,20 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
           if (!mbar_wait(fullA(s), par, abort) || !mbar_wait(fullS(s), par, abort)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t a0 = smem_u32(sA + s * stageA), b0 = smem_u32(sS + s * stageS);
-          {   // 4M with re in TMEM columns [0, Nt) and im in [256, 256 + Nt)
+          if constexpr (SPLIT) {
+            // Ar x [Sr; Si] -> (re, im) += (Ar Sr, Ar Si);  (-Ai) x [Si; -Sr] -> += (-Ai Si, Ai Sr)
+#pragma unroll
+            for (int ca = 0; ca < 2; ++ca) {
+#pragma unroll
+              for (int pi = 0; pi < M_::NPROD; ++pi) {
+                const int acc = M_::ta(pi) == 0 && M_::tb(pi) == 0 ? 0 : 1;   // hi x hi products: main
+                const uint64_t ad = smem_desc(a0 + (ca * TERMS + M_::ta(pi)) * kPlaneA);
+                const uint64_t bd = smem_desc(b0 + (3 * M_::tb(pi) + ca) * planeS);
+                mma<MODE>(tmem + (uint32_t)(acc * 256), ad, bd, ca ? idesc_n : idesc_p, started[acc] ? 1u : 0u);
+                started[acc] = true;
+              }
+            }
+          } else {   // 4M with re in TMEM columns [0, Nt) and im in [256, 256 + Nt)
 #pragma unroll
             for (int rp = 0; rp < 4; ++rp) {
               const int ca = (rp == 0 || rp == 2) ? 0 : 1;          // Ar, Ai, Ar, Ai
@@ -533,7 +618,8 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       const int64_t jg = jt * kRows + row;
       const bool valid = jg < a.J;
       float2* Cg = a.C + g * a.c_stride;
-      const int64_t p = valid ? jg / a.Sd : 0, sidx = valid ? jg % a.Sd : 0;
+      int64_t p, sidx;
+      split_row(a, jg, p, sidx);
       const int64_t jofs = p * a.NL * a.Sd + sidx;
       const int64_t strideNH = a.P * a.NL * a.Sd;
       if (my_last < 0) {
@@ -544,9 +630,20 @@ __global__ void __launch_bounds__(FastCfg<MODE>::THREADS, 1) cgemm_fast_kernel(c
       for (int ci = half; ci < nchunks; ci += 2) {
         const int c0 = ci * 16;
         float vr[16], vi[16];
-        tmem_ld16(tmem + lane_base + c0, vr);
-        tmem_ld16(tmem + lane_base + 256 + c0, vi);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (SPLIT) {
+          float sr[16], si[16];
+          tmem_ld16(tmem + lane_base + c0, vr);
+          tmem_ld16(tmem + lane_base + a.Nt + c0, vi);
+          tmem_ld16(tmem + lane_base + 256 + c0, sr);
+          tmem_ld16(tmem + lane_base + 256 + a.Nt + c0, si);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < 16; ++i) { vr[i] += sr[i]; vi[i] += si[i]; }
+        } else {
+          tmem_ld16(tmem + lane_base + c0, vr);
+          tmem_ld16(tmem + lane_base + 256 + c0, vi);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        }
         if (ci == my_last) {
           // last TMEM read of this tile by this warp: hand the columns back to the MMA
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1098,14 +1195,16 @@ __global__ void __launch_bounds__(128) split_site_kernel(const float2* S, int64_
   }
 }
 
+// Whether tiles of 128 rows do not straddle p unevenly and the inner extent of a tensor map's box
+// is at least 16 bytes.
+bool rows_fit_map(int64_t Sd) { return Sd >= 2 && (Sd % 128 == 0 || 128 % Sd == 0); }
+
 // Tensor map over B viewed as (s, k, p, item) 8-byte elements, box (box_s, ks, box_p, 1)
-// = one 128-row, ks-deep k-stage of a tile.  False if the shape does not allow it (the
-// box's inner extent must be at least 16 bytes: Sd >= 2; tiles must not straddle p
-// unevenly: Sd a multiple of 128 or a divisor of it).
+// = one 128-row, ks-deep k-stage of a tile.  False if the shape does not allow it.
 bool make_b_map(CUtensorMap* map, const void* B, int64_t b_stride, int batch, int64_t P, int64_t K,
                 int64_t Sd, int ks, int* box_s, int* box_p) {
   auto enc = tensor_map_encoder();
-  if (!enc || Sd < 2 || (Sd % 128 != 0 && 128 % Sd != 0)) return false;
+  if (!enc || !rows_fit_map(Sd)) return false;
   const int bs = (int)(Sd < 128 ? Sd : 128), bp = 128 / bs;
   const cuuint64_t dims[4] = {(cuuint64_t)Sd, (cuuint64_t)K, (cuuint64_t)P, (cuuint64_t)batch};
   const cuuint64_t item = (cuuint64_t)(batch > 1 ? b_stride : P * K * Sd) * 8;
@@ -1144,10 +1243,13 @@ int ensure_tc_attr() {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && !attr_done[dev]) {
-    using FC = FastCfg<MODE>;
-    using PC = PairCfg<MODE>;
-    cudaError_t e = cudaFuncSetAttribute(cgemm_fast_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    using FC = CtaCfg<MODE, false>;
+    using SC = CtaCfg<MODE, true>;
+    cudaError_t e = cudaFuncSetAttribute(cgemm_cta_kernel<MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)FC::smem(FC::NT_MAX));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(cgemm_cta_kernel<MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)SC::smem(SC::NT_MAX));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(cgemm_pair_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kMaxSmem - kStaticSmem);
@@ -1157,13 +1259,36 @@ int ensure_tc_attr() {
   return 0;
 }
 
+// Whether a default step takes tiles on one CTA.  With few k-steps a tile ends before the pair's
+// handshakes do (arrivals and commits that cross to the other SM, behind that tile's stores), and
+// the smaller tile without them is faster; with more, the pair's halved operand reads win.  us on
+// pairs / on one CTA, for about 10^6 columns in rows that a tensor map describes:
+//   TF32x3 K = 8, N = 32 143 / 71; K = 32, N = 64 207 / 165, N = 128 270 / 243; K = 48, N = 64 213 / 210,
+//     N = 128 286 / 289;
+//   BF16x2 K = 16, N = 64 163 / 105; K = 32, N = 64 169 / 133, N = 128 236 / 202; K = 48, N = 32 129 / 142;
+//   BF16x3 K = 16, N = 32 132 / 79, N = 128 240 / 201; K = 32, N = 64 183 / 149, N = 128 245 / 245; K = 48,
+//     N = 32 149 / 156;
+// and for 7 x 10^5 columns whose rows the producers load themselves, where a pair's 16 warps have
+// more loads in flight:
+//   TF32x3 K = 8, N = 32 96 / 61; K = 16, N = 16 87 / 88, N = 64 135 / 114; K = 24, N = 32 107 / 133;
+//   BF16x2 K = 16, N = 64 116 / 91; K = 32, N = 32 103 / 119; BF16x3 K = 16, N = 32 94 / 76, N = 128 177 / 179;
+//     K = 32, N = 32 107 / 113.
+template <int MODE>
+bool takes_cta_tile(int64_t K, int Nt, bool mapped) {
+  if (!mapped || K <= 16) return K <= 16;
+  return K <= 32 && (Mode<MODE>::TERMS == 2 || Nt <= 64);
+}
+
 template <int MODE>
 int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, int64_t b_stride, void* C,
                    int64_t c_stride, int64_t P, int64_t K, int64_t N, int64_t NL, int64_t Sd,
                    int batch, char* scratch, int64_t scratch_stride, int withhold, bool no_tma, int beta,
                    cudaStream_t st) {
   using M_ = Mode<MODE>;
-  const int64_t nt_max = fast ? FastCfg<MODE>::NT_MAX : PairCfg<MODE>::NT_MAX;
+  using FC = CtaCfg<MODE, false>;
+  using SC = CtaCfg<MODE, true>;
+  using PC = PairCfg<MODE>;
+  const int64_t nt_max = fast ? FC::NT_MAX : PC::NT_MAX;
   const int Nt = (int)(N < nt_max ? N : nt_max);   // N % 16 == 0
   const int KT = (int)(K / M_::KS);
   if (int err = ensure_tc_attr<MODE>()) return err;
@@ -1173,6 +1298,8 @@ int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, in
                                scratch_stride);
   count_launch();
   if (e != cudaSuccess) return (int)e;
+  const bool mapped = !fast && !no_tma && rows_fit_map(Sd);
+  const bool pair = !fast && !takes_cta_tile<MODE>(K, Nt, mapped);
   TcArgs a{};
   a.B = (const float2*)B; a.b_stride = b_stride;
   a.C = (float2*)C; a.c_stride = c_stride;
@@ -1180,7 +1307,7 @@ int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, in
   a.P = P; a.K = K; a.N = N; a.NL = NL; a.Sd = Sd; a.J = P * Sd;
   a.Nt = Nt;
   a.NHt = (int)(N / Nt);
-  const int rows = fast ? kRows : 2 * kRows;
+  const int rows = pair ? 2 * kRows : kRows;
   a.JT = (a.J + rows - 1) / rows;
   a.tiles = (int64_t)batch * a.JT * a.NHt;
   a.sd_shift = -1;
@@ -1188,24 +1315,23 @@ int launch_tc_mode(bool fast, const void* S, int64_t s_stride, const void* B, in
     if (Sd == int64_t(1) << b) a.sd_shift = b;
   a.withhold_s = withhold;
   a.beta = beta;
-  if (fast) {
-    const int64_t grid = a.tiles < num_sms() ? a.tiles : num_sms();
-    cgemm_fast_kernel<MODE><<<(unsigned)grid, FastCfg<MODE>::THREADS, FastCfg<MODE>::smem(Nt), st>>>(a);
-  } else {
-    alignas(64) CUtensorMap tmA;
-    std::memset(&tmA, 0, sizeof(tmA));
-    a.use_tma = !no_tma && make_b_map(&tmA, B, b_stride, batch, P, K, Sd, PairCfg<MODE>::SUB * M_::KS, &a.box_s, &a.box_p) ? 1 : 0;
+  alignas(64) CUtensorMap tmA;
+  std::memset(&tmA, 0, sizeof(tmA));
+  a.use_tma = mapped && make_b_map(&tmA, B, b_stride, batch, P, K, Sd, pair ? PC::SUB * M_::KS : M_::KS, &a.box_s, &a.box_p);
+  // the kernels start while split_site_kernel runs, so that barriers and launch latency (and for
+  // pairs the TMEM) are out of the way
+  if (pair) {
     const int64_t pairs = std::min<int64_t>(a.tiles, num_sms() / 2);
     pair_rings<MODE>(Nt, &a.stages, &a.nbuf);
-    // it starts while split_site_kernel runs, so that the pair's barriers, TMEM and launch
-    // latency are out of the way
-    e = launch_early(cgemm_pair_kernel<MODE>, dim3((unsigned)(2 * pairs)), dim3(PairCfg<MODE>::THREADS),
-                     PairCfg<MODE>::smem(Nt, a.stages, a.nbuf), st, a, tmA);
-    count_launch();
-    return (int)e;
+    e = launch_early(cgemm_pair_kernel<MODE>, dim3((unsigned)(2 * pairs)), dim3(PC::THREADS),
+                     PC::smem(Nt, a.stages, a.nbuf), st, a, tmA);
+  } else {
+    const unsigned grid = (unsigned)std::min<int64_t>(a.tiles, num_sms());
+    e = fast ? launch_early(cgemm_cta_kernel<MODE, false>, dim3(grid), dim3(FC::THREADS), FC::smem(Nt), st, a, tmA)
+             : launch_early(cgemm_cta_kernel<MODE, true>, dim3(grid), dim3(SC::THREADS), SC::smem(Nt), st, a, tmA);
   }
   count_launch();
-  return (int)cudaGetLastError();
+  return (int)e;
 }
 
 // ---- tensor-core rate probe -------------------------------------------------------

@@ -269,3 +269,24 @@ def test_bounded_wait_expires_on_many_pairs(qfx, prec, shape):
         out = qfx.contract_step(S, B, P, K, N, NL, Sd, precision=prec)
         qfx.sync()
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("prec,shape", [
+    ("tf32x3", (1, 8, 16, 16, 128)), ("tf32x3", (301, 8, 256, 128, 129)), ("tf32x3", (5, 16, 48, 24, 4100)),
+    ("tf32x3", (90, 32, 128, 128, 256)), ("tf32x3", (33, 40, 64, 64, 256)), ("tf32x3", (7, 24, 112, 112, 390)),
+    ("bf16x2", (3, 16, 384, 384, 1000)), ("bf16x2", (600, 32, 80, 80, 64)), ("bf16x2", (25, 48, 64, 64, 512)),
+    ("bf16x3", (130, 16, 16, 8, 1)), ("bf16x3", (700, 16, 128, 128, 62)), ("bf16x3", (9, 32, 64, 32, 2304)),
+    ("bf16x3", (9, 32, 96, 96, 2304))])
+def test_short_contractions(qfx, prec, shape):
+    """Few k-steps take tiles of 128 rows on one CTA, on both sides of the line to the pairs: one
+    tile and many a CTA, rows that a tensor map describes and rows that the producers load
+    (variant 13 has them loaded either way, and the bits are the same)."""
+    P, K, N, NL, Sd = shape
+    S = ri.random_complex((K, N), seed=31)
+    B = ri.random_complex((P, K, Sd), seed=32)
+    want = step_ref(S, B, P, K, N, NL, Sd)
+    dS, dB = torch.from_numpy(S.reshape(-1)).cuda(), torch.from_numpy(B.reshape(-1)).cuda()
+    got = [qfx.contract_step(dS, dB, P, K, N, NL, Sd, precision=prec, variant=v) for v in (-1, 13, -1)]
+    qfx.sync()
+    assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+    check_step(got[0].cpu().numpy().reshape(want.shape), want, S, B, P, K, N, NL, Sd, STEP_BOUND[prec])

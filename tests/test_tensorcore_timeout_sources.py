@@ -18,7 +18,7 @@ def ending(kernel):
     return body[body.rindex("\n  }\n\n") + 4:]      # roles close at this depth, before a blank line
 
 
-@pytest.mark.parametrize("kernel", ["cgemm_fast_kernel", "cgemm_pair_kernel"])
+@pytest.mark.parametrize("kernel", ["cgemm_cta_kernel", "cgemm_pair_kernel"])
 def test_mmas_end_before_tmem_is_freed(kernel):
     end = ending(kernel)
     dealloc = end.index("tcgen05.dealloc")
