@@ -7,8 +7,9 @@
 //   x BZ (consecutive values of one more axis) elements arrive by tensor-map copies with
 //   128-byte swizzle into a ring of shared buffers; each warp instruction then reads 16
 //   consecutive la by 2 consecutive lb (conflict-free under the swizzle) and writes two
-//   128-byte output segments; short output runs are lengthened by the axis next to la.  The input is viewed as a 5-D tensor: lb, la, and the
-//   other axes merged into at most three runs that are contiguous in the input.
+//   128-byte output segments; short output runs are lengthened by the axis next to la.  The
+//   input is viewed as a 5-D tensor: lb, la, and the other axes merged into at most three runs
+//   that are contiguous in the input.
 // - Otherwise a 32 x 32 tile goes through shared memory with plain loads, each block
 //   walking 8 consecutive batch coordinates.
 #include <cuda_runtime.h>
@@ -189,6 +190,7 @@ struct PermTma {
   int bx[3];                // box extent along each run (divides its innermost axis)
   int BZ, BY;               // box extents of the z run and of the run of the output axis next to la
   int y_outer;              // the y run is a later (slower) box dimension than the z run
+  int plain;                // la and lb are neighbours in the input and in the output
   int64_t ostr_z, ostr_y;   // output strides of those runs' innermost axes
   unsigned long long wait_ns;   // limit of every bounded wait
   int withhold;             // test hook: issue no copies (every consumer's wait runs out)
@@ -353,6 +355,7 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   a.Da = Da;
   a.Db = Db;
   a.ostr_b = f.ostr[lb];
+  a.plain = f.istr[la] == Db && f.ostr[lb] == Da;
   const int TA = Da >= 64 ? 64 : Da >= 32 ? 32 : 16;
   a.tiles_a = (Da + TA - 1) / TA;
   a.tiles_b = (Db + 15) / 16;
@@ -405,11 +408,11 @@ bool perm_tma_plan(const PermArgs& f, const void* in, PermTma* t, CUtensorMap* m
   a.ostr_z = a.ostr_y = 0;
   // Boxes of 8 KB or more.  Where la fills one tile of 16 or 32, an output run is 128 or 256
   // bytes; the output axis next to it, ly, then becomes a run of its own and is boxed 4 (or 2)
-  // deep, and the run that is innermost in the input lengthens the reads.  2^27 elements, GB/s, with
-  // four buffers a block (two give more, launch_perm_tma):
-  // seven axes reversed, la = 16: 5020 with 8 values of run 0 instead, 6090 with 4 of ly and 2 of
-  // the last run, 6040 with 2 and 4, 5170 with 8 and 1; la = 32: 4890, and 5940 with 2 and 2 (4
-  // and 1: 5670).  Otherwise the box takes several values of run 0's innermost axis.
+  // deep, and the run that is innermost in the input lengthens the reads.  2^27 elements, GB/s: seven
+  // axes reversed, la = 16: 5100 with 8 values of run 0 instead, 6310 with 4 of ly and 2 of the last
+  // run, 6370 with 2 and 4, 5920 with 8 and 1; (16, 4096, 16, 128) reversed 5100, 6140, 6040, 6190; la = 32,
+  // (32, 8, 32, 16, 8, 8, 16) reversed: 5440, and 6330 with 2 and 2 (4 and 1: 6120).  Otherwise the box
+  // takes several values of run 0's innermost axis.
   int rz = -1, ry = -1;
   const int ly = Da == TA && TA < 64 && la >= 1 && la - 1 != lb && f.dim[la - 1] % 2 == 0 ? la - 1 : -1;
   if (ly >= 0 && cut_runs(ly, &ry)) {
@@ -474,19 +477,30 @@ int launch_perm_tma(const PermTma& a, const CUtensorMap& map, float2* out, cudaS
   int sms = 0, l2 = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev0);
   cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev0);
-  // Blocks per SM, with two buffers each: tensors beyond L2 take four.  More copies in flight
-  // crowd the stores, fewer leave the memory idle.  2^27 elements (2^28 for the square), GB/s with
-  // 3 / 4 / 6 / 8 blocks, then 4 buffers and as many blocks as fit: seven axes reversed 5560 /
-  // 6300 / 5370 / 5370, 5550; 16384 x 16384 5930 / 6590 / 5180 / 5110, 5020; (16, 4096, 16, 128)
-  // reversed 5920 / 6200 / 5260 / 5250, 5350.  Tiles cut off at the edge of la or lb copy less
-  // and take more blocks for the same bytes: (64, 2, 89, 69, 32), half of whose tiles are 5 of 64
-  // wide, 3070 / 3670 / 4180 / 4530, 4620.  What L2 holds, or nearly, is bound by latency and
-  // takes eight; us with 4 / 6 / 8: (512, 106, 128) 22.6 / 19.9 / 18.5, 8192 x 1024 (134 MB in
-  // and out) 26.6 / 23.7 / 22.6; but 4096 x 4096 (268 MB) 46.9 / 51.9 / 53.4.  220 KB of shared
-  // memory are the limit, which six blocks of 16 KB boxes fill.
-  const int64_t tile_el = a.tiles_a * a.tiles_b * TA * 16, real_el = a.Da * a.Db;
+  // Blocks per SM: more copies in flight crowd the stores, fewer leave the memory idle.  us with 4 /
+  // 6 / 8 blocks of two buffers, then with four buffers and as many blocks as fit (220 KB of shared
+  // memory are the limit):
+  //  - boxes of 8 KB take 4 where the output runs along la are long, and where la and lb are neighbours
+  //    in input and output, a batch of plain transposes: 16384 x 16384 651 / 836 / 847, 853; (64, 2^20)
+  //    173 / 187 / 195, 200;
+  //  - 6 where they are short (one tile of la, or two of 64): (27, 8, 64, 65, 16) to (0, 4, 1, 3, 2) 47 /
+  //    41 / 42, 44; (32, 64, 128, 64) to (2, 0, 3, 1) 54 / 47 / 50, 52;
+  //  - boxes of 16 KB take 4: seven axes reversed 340 / 400 / 400, 387;
+  //  - boxes below 8 KB (no axis with a factor 2 to box) need four buffers and all the blocks: (25,
+  //    32, 47, 2, 16, 32) to (3, 5, 1, 0, 2, 4) 155 / 127 / 111, 107; (4194304, 16) 324 / 247 / 214, 164;
+  //  - tiles cut off at the edge of la or lb copy less and take more blocks for the same bytes: (64, 2,
+  //    89, 69, 32) reversed, half of whose tiles are 5 of 64 wide, 113 / 99 / 92, 90; but not where la
+  //    has 16-wide tiles, whose short runs crowd the stores already: (64, 18, 64, 16, 32) to (0, 2, 3, 4,
+  //    1) 141 / 162 / 163, 153;
+  //  - what L2 holds, or nearly, is bound by latency and takes 8: (512, 106, 128) 22.6 / 19.9 / 18.5,
+  //    8192 x 1024 (134 MB in and out) 26.6 / 23.7 / 22.6; but 4096 x 4096 (268 MB) 46.9 / 51.9 / 53.4.
+  const int64_t tile_el = (TA > 16 ? a.tiles_a * TA : a.Da) * a.tiles_b * 16, real_el = a.Da * a.Db;
   const bool in_l2 = 16 * real_el * a.nbatch * a.BZ * a.BY <= (int64_t)l2 * 3 / 2;
-  int64_t per_sm = in_l2 ? 8 : std::min((4 * tile_el + real_el - 1) / real_el, (int64_t)8);
+  const int box = 16 * TA * 8 * a.BZ * a.BY;
+  const bool short_runs = box == 8192 && a.Da <= (TA == 64 ? 128 : TA) && !a.plain;
+  int64_t per_sm = 8;
+  if (box >= 8192 && !in_l2)
+    per_sm = std::min(short_runs ? 6 * tile_el / real_el : (4 * tile_el + real_el - 1) / real_el, (int64_t)8);
   per_sm = std::min(per_sm, (int64_t)((220u << 10) / (smem + 512)));
   const int64_t want = (int64_t)(sms > 0 ? sms : 1) * per_sm;
   const unsigned grid = (unsigned)(a.total < want ? a.total : want);
@@ -553,11 +567,15 @@ int launch_permute(const void* in, void* out, int rank, const int64_t* shape,
         g_perm_withhold_ns = 0;
       }
       const bool y = tp.BY > 1;
-      const int err = TA == 64 ? launch_perm_tma<64, 2, false>(tp, map, dst, st)
-                    : TA == 32 ? (y ? launch_perm_tma<32, 2, true>(tp, map, dst, st)
-                                    : launch_perm_tma<32, 2, false>(tp, map, dst, st))
-                               : (y ? launch_perm_tma<16, 2, true>(tp, map, dst, st)
-                                    : launch_perm_tma<16, 2, false>(tp, map, dst, st));
+      const bool small = 16 * TA * 8 * tp.BZ * tp.BY < 8192;   // see launch_perm_tma
+      const int err = TA == 64   ? launch_perm_tma<64, 2, false>(tp, map, dst, st)
+                      : TA == 32 ? (y       ? launch_perm_tma<32, 2, true>(tp, map, dst, st)
+                                    : small ? launch_perm_tma<32, 4, false>(tp, map, dst, st)
+                                            : launch_perm_tma<32, 2, false>(tp, map, dst, st))
+                      : y        ? (small ? launch_perm_tma<16, 4, true>(tp, map, dst, st)
+                                          : launch_perm_tma<16, 2, true>(tp, map, dst, st))
+                                 : (small ? launch_perm_tma<16, 4, false>(tp, map, dst, st)
+                                          : launch_perm_tma<16, 2, false>(tp, map, dst, st));
       count_launch();
       return err;
     }

@@ -350,6 +350,19 @@ def test_permute_short_output_runs(qfx, case):
     np.testing.assert_array_equal(out.cpu().numpy(), primitives.permute(x, shape, perm).reshape(-1))
 
 
+@pytest.mark.parametrize("case", [((301, 5, 32, 34), (0, 1, 3, 2)), ((32, 18), (1, 0)), ((40011, 32), (1, 0)),
+                                  ((1201, 16, 18), (0, 2, 1)), ((65537, 16), (1, 0)), ((5, 48, 333, 20), (3, 1, 2, 0)),
+                                  ((34, 301, 16, 20), (3, 1, 0, 2)), ((6, 3, 16, 16), (3, 1, 0, 2))])
+def test_permute_small_boxes(qfx, case):
+    """Tensor-map transposes with no axis of even extent to box beside la and lb (boxes of 2 and 4
+    KB, by fours in the ring): one tile and more than all buffers of the GPU hold at once."""
+    shape, perm = case
+    x = ri.random_complex(int(np.prod(shape)), seed=7)
+    out = qfx.permute(torch.from_numpy(x).cuda(), shape, perm)
+    qfx.sync()
+    np.testing.assert_array_equal(out.cpu().numpy(), primitives.permute(x, shape, perm).reshape(-1))
+
+
 @pytest.mark.parametrize("case", [((4, 5, 6), (2, 0, 1)), ((33, 65), (1, 0)),
                                   ((2, 3, 4, 5, 6), (4, 2, 0, 3, 1)), ((7, 8, 9), (0, 2, 1)),
                                   ((64, 3, 64), (2, 1, 0)), ((5, 1, 7), (1, 2, 0)),
