@@ -43,8 +43,8 @@ uint64_t a256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 // ---- seed: R_n[f(o)] = gbar[o] * 2^-m ------------------------------------------------
 __global__ void __launch_bounds__(kT) seed_kernel(const double* gout, const int32_t* __restrict__ open_perm,
                                                   int n_open, float2* R, int* m_out) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ double red[kT];
   const int64_t per = int64_t(1) << n_open;
   double mx = 0.0;
@@ -70,8 +70,8 @@ __global__ void __launch_bounds__(kT) seed_kernel(const double* gout, const int3
 template <int BM>
 __global__ void __launch_bounds__(kT) rstep_kernel(const float2* S, const float2* Rin, float2* Rout, int64_t P, int64_t K,
                                                    int64_t N, int64_t NL, int64_t Sd) {
-  launch_next();
   launch_wait();
+  launch_next();
   constexpr int BJ = 64, BR = 16, TMK = BM / 16;
   static_assert(kT == 256 && (BM == 16 || BM == 64), "thread layout");
   __shared__ float2 As[BR][BM + 1];
@@ -157,8 +157,8 @@ struct ConjTable {
   int32_t count;
 };
 __global__ void __launch_bounds__(kT) conj_transpose_kernel(const float2* sites, float2* sconj, const ConjTable tab) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ float2 tile[32][33];
   const int y = blockIdx.y;
   const int64_t K = tab.K[y], N = tab.N[y];
@@ -208,8 +208,8 @@ __device__ __forceinline__ void g_cp_async8(void* smem, const void* gmem, bool p
 template <int BM, int BN>
 __global__ void __launch_bounds__(kT) grads_kernel(const float2* Lin, const float2* Rin, float2* part, int64_t P, int64_t K,
                                                    int64_t N, int64_t NL, int64_t Sd, int64_t chunk) {
-  launch_next();
   launch_wait();
+  launch_next();
   constexpr int BJ = 16, TMK = BM / 16, TNN = BN / 16;
   constexpr int LA = BM + 2, LB = BN + 2;   // rows of 16-byte multiples, 2-way store conflicts
   static_assert(kT == 256 && BM % 16 == 0 && BN % 16 == 0, "thread layout");
@@ -341,8 +341,8 @@ int launch_grads(const GradsGeom& g, const float2* Lin, const float2* Rin, float
 // butterfly adds the lanes (deterministic).
 __global__ void __launch_bounds__(kT) reduce_chunks_kernel(const float2* part, int64_t chunks,
                                                            int64_t KN, float2* out) {
-  launch_next();
   launch_wait();
+  launch_next();
   const int64_t t = ((int64_t)blockIdx.x * kT + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= KN) return;   // warp-uniform: t is the same for all lanes of a warp
@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(kT) fold_backward_kernel(
     const FoldSite* __restrict__ sites, const FoldEvent* __restrict__ events, const float* __restrict__ matsf,
     const CutDev* __restrict__ cuts, int n_cuts, const uint64_t* x1w, int64_t sid,
     const float2* sgrad, double* bpart, const int64_t* __restrict__ part_off) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ double wpart[kT / 32][kMaxEvents][8];
   const FoldSite st = sites[blockIdx.y];
   const int nev = st.ev_end - st.ev_begin;
@@ -547,8 +547,8 @@ __global__ void __launch_bounds__(kT) event_reduce_kernel(const FoldSite* __rest
                                                           const int64_t* __restrict__ part_off,
                                                           const int* hdr_exps, const int* m_ptr,
                                                           int n_events, double* evgrad) {
-  launch_next();
   launch_wait();
+  launch_next();
   const int t = blockIdx.x * kT + threadIdx.x;
   if (t >= n_events * 32) return;
   const int e = t / 32, entry = t % 32;
@@ -581,8 +581,8 @@ __global__ void __launch_bounds__(kT) gate_accum_kernel(const int32_t* __restric
                                                         const FoldEvent* __restrict__ events, int n_gates,
                                                         int per_gate, const double* evgrad,
                                                         double* grad) {
-  launch_next();
   launch_wait();
+  launch_next();
   const int t = blockIdx.x * kT + threadIdx.x;
   if (t >= n_gates * 2 * per_gate) return;
   const int gte = t / (2 * per_gate), ent = t % (2 * per_gate), ce = ent / 2, ri = ent & 1;

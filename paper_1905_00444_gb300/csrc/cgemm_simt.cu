@@ -22,8 +22,8 @@ __device__ __forceinline__ void simt_cp_async8(float2* smem, const float2* gmem)
 
 template <int BM, int BJ, int TM, int TJ, bool KMODE>
 __global__ void __launch_bounds__(256, 2) cgemm_step_kernel(const StepArgs a) {
-  launch_next();
   launch_wait();
+  launch_next();
   extern __shared__ float4 smem_raw[];
   cgemm_tile<BM, BJ, TM, TJ, KMODE>(a, blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -68,8 +68,8 @@ int launch_cfg(const StepArgs& a, int batch, cudaStream_t stream) {
 constexpr int kPartsOut = 256;
 __global__ void __launch_bounds__(kPartsOut) small_parts_kernel(const float2* S, const float2* B, float2* part, int chunk,
                                                                int64_t parts, int N, int Sd, int KB) {
-  launch_next();
   launch_wait();
+  launch_next();
   extern __shared__ __align__(16) float2 slab[];
   const int out = N * Sd, per_block = kPartsOut / out, row = N + Sd;
   const int own = threadIdx.x / out, e = threadIdx.x - own * out, n = e / Sd, s = e - n * Sd;
@@ -121,8 +121,8 @@ template <int E>
 __global__ void __launch_bounds__(E * kRedL) reduce_parts_kernel(const float2* part,
                                                                  int64_t part_stride, int64_t parts,
                                                                  int64_t out, float2* C, int64_t c_stride) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ double2 lanes[kRedL][E];
   const int el = threadIdx.x % E, lane = threadIdx.x / E;
   const int64_t e = (int64_t)blockIdx.x * E + el;

@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(CtaCfg<MODE, SPLIT>::THREADS, 1)
     }
     mbar_init_fence();
   }
-  launch_next();
   launch_wait();       // the site image is written; before the TMEM, which an earlier kernel may hold
+  launch_next();
   __syncwarp();
   if (warp == 12) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_base_slot))
@@ -833,8 +833,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   cluster_barrier();   // barriers of both CTAs initialised, TMEM allocated in both
-  launch_next();
   launch_wait();       // the site image is written
+  launch_next();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_slot;
   volatile int* abort = &abort_flag;
@@ -1163,8 +1163,8 @@ __global__ void __launch_bounds__(128) split_site_kernel(const float2* S, int64_
                                                           int64_t img_stride) {
   using M_ = Mode<MODE>;
   constexpr int TERMS = M_::TERMS, KS = M_::KS;
-  launch_next();
   launch_wait();
+  launch_next();
   const int n = blockIdx.x * 128 + threadIdx.x;
   const int ks = blockIdx.y;
   const int g = blockIdx.z;

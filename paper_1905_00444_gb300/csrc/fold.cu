@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(
     const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
     int64_t item0, char* hdr, uint64_t hdr_stride, char* items, uint64_t item_bytes,
     uint64_t sites_off, int n_sites) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ foldk::FoldStage sm;
   const FoldSite st = sites[blockIdx.y];
   const int g = blockIdx.z;
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kSmallSite) fold_scale_kernel(
     const uint64_t* x1, int x1_words, int64_t n_batch, int64_t slice_begin,
     int64_t item0, char* hdr, uint64_t hdr_stride, char* items, uint64_t item_bytes,
     uint64_t sites_off, int n_sites) {
-  launch_next();
   launch_wait();
+  launch_next();
   __shared__ foldk::FoldStage sm;
   __shared__ unsigned largest;
   const FoldSite st = sites[blockIdx.x];
@@ -125,8 +125,8 @@ __global__ void __launch_bounds__(kSmallSite) fold_scale_kernel(
 __global__ void __launch_bounds__(kThreads) scale_kernel(
     const FoldSite* __restrict__ sites, char* hdr, uint64_t hdr_stride, char* items,
     uint64_t item_bytes, uint64_t sites_off, int n_sites) {
-  launch_next();
   launch_wait();
+  launch_next();
   const FoldSite st = sites[blockIdx.y];
   const int g = blockIdx.z;
   const unsigned* maxabs = reinterpret_cast<const unsigned*>(hdr + (uint64_t)g * hdr_stride);
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(kThreads) accumulate_kernel(
     const int32_t* __restrict__ open_perm, int n_open, int n_sites, int64_t n_batch,
     int64_t item0, int items, const char* hdr, uint64_t hdr_stride, const char* itemsp,
     uint64_t item_bytes, uint64_t final_off, double* out) {
-  launch_next();
   launch_wait();
+  launch_next();
   const int64_t per = int64_t(1) << n_open;
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= n_batch * per) return;

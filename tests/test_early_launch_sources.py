@@ -56,3 +56,13 @@ def test_restrict_is_for_tables_only(kernel):
         if "__restrict__" in param:
             kind, name = re.fullmatch(r"\s*const\s+(\w+)\s*\*\s*__restrict__\s+(\w+)\s*", param).groups()
             assert name in TABLES.get(kind, ()), param
+
+
+@pytest.mark.parametrize("kernel", early_kernels(), ids=lambda k: k[0])
+def test_successors_start_behind_the_wait(kernel):
+    """A kernel that lets its successor start before its own wait lets the whole chain become
+    resident at once, which crowds the blocks of small grids onto some of the SMs."""
+    body = kernel[2]
+    assert body.count("launch_wait()") == 1
+    if "launch_next()" in body:
+        assert body.index("launch_wait()") < body.index("launch_next()")
