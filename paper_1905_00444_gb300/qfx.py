@@ -6,7 +6,6 @@ fallback path.
 from __future__ import annotations
 
 import ctypes as C
-import operator
 import os
 import re
 from typing import Iterable, List, Optional, Sequence
@@ -150,7 +149,6 @@ def launch_count() -> int:
 GATE_DTYPE = np.dtype([("layer", np.int32), ("q0", np.int32), ("q1", np.int32), ("kind", np.int32),
                        ("mat", np.complex128, 16)])
 assert GATE_DTYPE.itemsize == C.sizeof(Gate)
-_FIELDS = operator.attrgetter("layer", "q0", "q1", "kind")
 
 
 def gate_table(gates, mats):
@@ -160,11 +158,12 @@ def gate_table(gates, mats):
     table = np.zeros(max(1, len(gates)), dtype=GATE_DTYPE)
     if not gates:
         return table
-    for name, column in zip(("layer", "q0", "q1", "kind"), zip(*map(_FIELDS, gates))):
-        # what is not integers of 32 bits goes through the ABI's own type, which refuses or wraps it
+    for name, column in zip(("layer", "q0", "q1", "kind"),
+                            zip(*[(g.layer, g.q0, g.q1, g.kind) for g in gates])):
+        # what is not integers of 32 bits (a sum with others is not an integer either) goes through
+        # the ABI's own type, which refuses or wraps it
         try:
-            plain = all(issubclass(t, (int, np.integer)) for t in set(map(type, column)))
-            table[name] = column if plain else [C.c_int32(v).value for v in column]
+            table[name] = column if isinstance(sum(column), (int, np.integer)) else [C.c_int32(v).value for v in column]
         except OverflowError:
             table[name] = [C.c_int32(v).value for v in column]
     if isinstance(mats, np.ndarray):
