@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(CtaCfg<MODE, SPLIT>::THREADS, 1)
             int l = nl;
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              o[i] = *d;
+              o[i] = __ldcg(d);
               d += a.Sd;
               if (++l == NL) { l = 0; d += strideNH - (int64_t)NL * a.Sd; }
             }
@@ -1102,7 +1102,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
             int l = left;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              o[e] = *d;
+              o[e] = __ldcg(d);
               d += a.Sd;
               if (--l == 0) { l = NL; d += wrap; }
             }
