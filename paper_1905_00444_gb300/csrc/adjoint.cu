@@ -721,7 +721,7 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
   const int64_t n_items = (slice_end - slice_begin) * n_batch;
   auto step_fwd = [&](int i, const char* in, char* out) -> int {
     const Step& sp = p->steps[i];
-    const int v = fill_variant(pick_variant(sp.N, sp.Sd), sp.N, sp.P * sp.Sd, 1);
+    const int v = fill_variant(pick_variant(sp.N, sp.Sd), sp.K, sp.N, sp.P * sp.Sd, 1);
     return launch_step(site_ptr(sp.site), 0, in, 0, out, 0, sp.P, sp.K, sp.N, sp.NL, sp.Sd, 1, v,
                        QFX_PREC_FP32_SIMT, st);
   };
@@ -794,7 +794,7 @@ qfx_status backward(const qfx_plan* p, const uint64_t* x1, int64_t n_batch, int6
       if (err2) return cuda_fail(err2, "qfx_amplitudes_backward: site gradient");
       float2* Rnext = (float2*)rr(rsel ^ 1);
       if (use_conj[i]) {
-        const int v = fill_variant(pick_variant(sp.K, sp.Sd), sp.K, J, 1);
+        const int v = fill_variant(pick_variant(sp.K, sp.Sd), sp.N, sp.K, J, 1);
         err2 = launch_step(sconj + p->sites[sp.site].offset, 0, Rcur, 0, Rnext, 0, sp.P, sp.N, sp.K,
                                      sp.K, sp.Sd, 1, v, QFX_PREC_FP32_SIMT, st);
         if (err2) return cuda_fail(err2, "qfx_amplitudes_backward: reverse step");

@@ -207,32 +207,42 @@ int num_sms() {
   return n[dev] > 0 ? n[dev] : 1;
 }
 
-// Variants 0..9 keep their tile when its grid gives more than three CTAs to two SMs: two of
-// them share an SM, and the fill tiles, with more reads of shared memory per product, gain
-// nothing (8 x 4096 columns, K = N = 64, 256 CTAs: 28.7 us against 28.8; 65536 columns of
-// K = 256, N = 16, 256 CTAs: 72 against 80; but 208 CTAs, K = 1024, N = 512: 351 against 282).
-// On a smaller grid a tile's time is the latency of its k loop, the less the fewer products it
-// has: the step takes the first of the fill tiles below, in this order, that gives more CTAs
-// than SMs, or else the one that gives most (852 columns of K = 1024, N = 512: 345 us with 64 x
-// 128, 195 with 64 x 64, 135 with 16 x 128).  Every tile sums an output's k terms in the same
-// order, so the choice never changes a result.
-int fill_variant(int variant, int64_t N, int64_t J, int batch) {
-  struct Tile { int bm, bj; };
-  static const Tile base[5] = {{128, 64}, {64, 128}, {32, 256}, {16, 256}, {8, 512}};
-  static const Tile fill[5] = {{64, 64}, {32, 128}, {16, 128}, {8, 256}, {8, 128}};   // 20..24, 25..29
+// Variants 0..9 keep their tile when its grid gives more than three CTAs to two SMs (8 x 4096
+// columns, K = N = 64, 256 CTAs: 25.9 us, 26.0 with 64 x 64).  A smaller grid is bound by the latency
+// of a tile's k loop, and the CTAs that share an SM take about as long as one after another: the
+// step takes the tile of least time.  A tile's times, alone on its SM and for each of those that
+// share one, are relative to 64 x 64 alone (105 us at K = 1024 and even Sd, 117 odd), for even and for
+// odd Sd; they are fitted to 1300 steps of K = 16 to 1024, N = 2 to 512, 64 to 80000 columns.  The
+// choice is 0.6% slower than each step's fastest tile on geometric mean, and 11% faster than the
+// first tile that gives more CTAs than SMs (852 columns of K = 1024, N = 512: 106 us with 32 x 128 and
+// 112 CTAs, 136 with 16 x 128 and 224).  Where K < 32 loads and stores count more than the loop, and
+// CTAs that share an SM hide one another's: their times count 0.65 (all amplitudes of 4x4x(1+16+1)
+// 110.7 us, 113.4 without).
+// Every tile sums an output's k terms in the same order, so the choice never changes a result.
+int fill_variant(int variant, int64_t K, int64_t N, int64_t J, int batch) {
+  struct Tile { int bm, bj, alone[2], shared[2]; };
+  static const Tile base[5] = {{128, 64, {180, 220}, {172, 172}}, {64, 128, {180, 220}, {172, 172}},
+                               {32, 256, {217, 217}, {200, 200}}, {16, 256, {120, 140}, {125, 125}},
+                               {8, 512, {145, 193}, {180, 180}}};
+  static const Tile fill[5] = {{64, 64, {100, 100}, {97, 97}}, {32, 128, {102, 102}, {107, 107}},    // 20..24, 25..29
+                               {16, 128, {72, 72}, {74, 68}}, {8, 256, {85, 112}, {97, 80}},
+                               {8, 128, {53, 53}, {60, 54}}};
   if (variant < 0 || variant > 9 || batch < 1) return variant;
-  auto ctas = [&](const Tile& t) { return ((N + t.bm - 1) / t.bm) * ((J + t.bj - 1) / t.bj) * batch; };
   const int64_t sms = num_sms();
-  int64_t most = ctas(base[variant % 5]);
-  if (2 * most > 3 * sms) return variant;
+  const int odd = variant >= 5;
+  auto ctas = [&](const Tile& t) { return ((N + t.bm - 1) / t.bm) * ((J + t.bj - 1) / t.bj) * batch; };
+  auto time = [&](const Tile& t) {
+    const int64_t on_sm = (ctas(t) + sms - 1) / sms;
+    return on_sm == 1 ? (int64_t)t.alone[odd] : on_sm * t.shared[odd] * (K < 32 ? 65 : 100) / 100;
+  };
+  const Tile& own = base[variant % 5];
+  int64_t least = time(own);
+  if (2 * ctas(own) > 3 * sms) return variant;
   int best = variant;
   for (int i = 0; i < 5; ++i) {
-    if (fill[i].bm > base[variant % 5].bm) continue;
-    const int64_t c = ctas(fill[i]);
-    if (c <= most) continue;
-    most = c;
-    best = 20 + i + (variant >= 5 ? 5 : 0);
-    if (c > sms) break;
+    if (fill[i].bm > own.bm || time(fill[i]) >= least) continue;
+    least = time(fill[i]);
+    best = 20 + i + 5 * odd;
   }
   return best;
 }

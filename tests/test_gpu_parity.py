@@ -335,6 +335,21 @@ def test_smallest_fill_tile(qfx, shape):
     qfx.sync()
 
 
+@pytest.mark.parametrize("shape", [(213, 64, 512, 256, 4), (40, 40, 99, 33, 7), (1, 33, 2, 1, 64), (19, 32, 16, 16, 1024),
+                                   (7142, 32, 3, 3, 7), (2, 48, 17, 17, 6000), (30, 31, 64, 64, 128), (30, 32, 64, 64, 128),
+                                   (1, 36, 130, 130, 2049), (11, 64, 64, 32, 3000)])
+def test_tile_of_a_small_grid(qfx, shape):
+    """The tile that a step takes on a grid below 1.5 CTAs per SM, by the length of its k loop and
+    the CTAs that would share an SM: the bits of every tile, partial tiles of rows and columns."""
+    P, K, N, NL, Sd = shape
+    S = torch.from_numpy(ri.random_complex(K * N, seed=14)).cuda()
+    B = torch.from_numpy(ri.random_complex(P * K * Sd, seed=15)).cuda()
+    auto = qfx.contract_step(S, B, P, K, N, NL, Sd).cpu().numpy()
+    for v in (6, 8, 25, 26, 27, 28) + ((1, 20, 21, 22, 23) if Sd % 2 == 0 else ()):
+        np.testing.assert_array_equal(auto, qfx.contract_step(S, B, P, K, N, NL, Sd, variant=v).cpu().numpy())
+    qfx.sync()
+
+
 @pytest.mark.parametrize("case", [((16, 8, 3, 16), (3, 2, 1, 0)), ((16, 6, 5, 40), (3, 2, 1, 0)),
                                   ((16, 4, 24), (2, 1, 0)), ((32, 2, 7, 18), (3, 2, 1, 0)),
                                   ((2, 16, 3, 4, 32), (4, 2, 0, 3, 1)), ((4, 2, 32, 5, 16), (3, 4, 1, 0, 2)),
