@@ -28,17 +28,24 @@ __global__ void __launch_bounds__(256, 2) cgemm_step_kernel(const StepArgs a) {
   cgemm_tile<BM, BJ, TM, TJ, KMODE>(a, blockIdx.x, blockIdx.y, smem_raw);
 }
 
+// A grid of at most one CTA per SM asks for more than half of an SM's shared memory, so that no two
+// of its CTAs share an SM.  Such a grid is chosen for it (fill_variant), but CTAs that start early
+// take the slots that the kernel before leaves, two on some SMs, and then the step takes twice its
+// time: K = 128, N = 64 over 16384 columns in 128 CTAs behind K = 64 in 256 47 us, and 26 so; a call of
+// 6x5x(1+28+1) 923 us and 684.
+constexpr size_t kOwnSm = 116 << 10;
+
 // Shared-memory opt-in of one tile kernel, once per device (also called ahead of a graph
 // capture, which must not be the first launch to set it).
 template <int BM, int BJ, int TM, int TJ, bool KMODE>
 int ensure_attr() {
-  using C_ = Cfg<BM, BJ, TM, TJ, KMODE>;
+  static_assert(Cfg<BM, BJ, TM, TJ, KMODE>::SMEM <= kOwnSm, "a tile fits its request");
   static int attr_done[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && !attr_done[dev]) {
     cudaError_t e = cudaFuncSetAttribute(cgemm_step_kernel<BM, BJ, TM, TJ, KMODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C_::SMEM);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOwnSm);
     if (e != cudaSuccess) return (int)e;
     attr_done[dev] = 1;
   }
@@ -55,7 +62,8 @@ int launch_cfg(const StepArgs& a, int batch, cudaStream_t stream) {
   const int64_t blocks = NT * JT;
   if (blocks > 0x7fffffffLL || batch > 65535) return (int)cudaErrorInvalidConfiguration;
   count_launch();
-  return (int)launch_early(kern, dim3((unsigned)blocks, batch), dim3(256), C_::SMEM, stream, a);
+  const size_t smem = blocks * batch <= num_sms() ? kOwnSm : C_::SMEM;
+  return (int)launch_early(kern, dim3((unsigned)blocks, batch), dim3(256), smem, stream, a);
 }
 
 // Chunk products of a split-K contraction with a small result: part c is the N x Sd product
