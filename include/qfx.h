@@ -362,7 +362,8 @@ qfx_status qfx_tensor_peak(int32_t precision, int64_t mmas_per_sm, double* tflop
  * 16-byte aligned, no aliasing.  `variant` < 0 lets the library choose (FP32 only);
  * FP32 tile variants are 0-9 (0-4 need an even Sd) and their fill variants 20-23 (even
  * Sd) and 25-28, which compute 4096 or 2048 outputs per CTA for grids that would leave SMs
- * idle; every variant gives bit-identical results.
+ * idle; every variant gives bit-identical results.  The library's own choice may also be the
+ * fill tile of 8 rows, 24 or 29, which profile records then name; it cannot be asked for.
  * Tensor-core precisions run on tcgen05 when N % 16 == 0 and N <= 128 or a multiple of 128
  * (fast accumulation: N <= 256 or a multiple of 256), K a multiple of the term's k step
  * (16 for BF16x3 and BF16x2, 8 for TF32x3) and P*Sd >= 128, otherwise on the FP32
@@ -414,7 +415,7 @@ qfx_status qfx_frugal_select(const qfx_plan* p, const uint64_t* x1, int64_t n_ba
  * contraction-step launch is bracketed by CUDA events on its own stream. */
 typedef struct {
   int32_t step;       /* plan step index, or -1 for qfx_contract_step */
-  int32_t variant;
+  int32_t variant;    /* a plan step's own variant; of qfx_contract_step, the one that ran */
   int32_t kind;       /* 0 = contraction step, 1 = fold, 2 = scale, 3 = accumulate,
                          4 = permute, 5 = frugal select */
   float ms;

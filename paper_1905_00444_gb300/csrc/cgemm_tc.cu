@@ -253,10 +253,14 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
-// Arrives on the barrier at this shared-memory offset in CTA 0 of the pair.  What it stands
-// for is ordered by itself (planes by the writers' proxy fences, TMEM reads by the tcgen05
-// fence), so the default scope is enough: a release at cluster scope waits for all of the
-// thread's stores, those of C among them, and made a k-stage take 2400 clk or more.
+// Arrives on the barrier at this shared-memory offset in CTA 0 of the pair.  The planes that it
+// stands for are ordered by their writers' proxy fences, the TMEM reads by the tcgen05 fence.  Its
+// own order is the default one, a release within the CTA: that the other CTA sees what lies before
+// it rests on the customary use of this form for CTA pairs and on tests that compare every bit, not
+// on the memory model's words.  Release and acquire at cluster scope wait for the thread's other
+// stores, those of C among them.  us with the default / with cluster scope in the producers / in all
+// arrivals and waits: BF16x3 K = N = 256 over 2^19 columns 876 / 928 / 978, K = N = 64 over 2^21 406 /
+// 528 / 548, TF32x3 K = N = 256 866 / 970 / 1002, a BF16x2 chunk of K = 1024 473 / 781 / 790.
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
   asm volatile(
       "{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, 0;\n"
@@ -900,8 +904,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
         in.step(nbuf);
       }
     } else {
-      // rows that no tensor map describes: loads issued one k-stage ahead into registers (plain
-      // ones: the kernel that writes B may still run when this one starts)
+      // rows that no tensor map describes: loads issued one k-stage ahead into registers (not
+      // the read-only path: the kernel that writes B may still run when this one starts)
       float2 nxt[SUB][KH];
       int64_t t = pair0;
       int it = 0;
@@ -1094,9 +1098,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE>::THREA
           int left = (nh0 + 1) * NL - n0;   // columns to the end of this nh
           float2* dst = Cj + nh0 * wrap + (int64_t)n0 * a.Sd;
           if (a.beta) {   // a chunk of a long contraction: add into C
-            // all 8 reads first: one memory latency per chunk, not one per element.  Plain
-            // loads: the launch of the chunk before may still be writing C while this one
-            // starts, and the read-only path is for memory that nothing writes meanwhile
+            // all 8 reads first: one memory latency per chunk, not one per element.  Not the
+            // read-only path, which is for memory that nothing writes during the kernel: this
+            // kernel writes C, and the one of the chunk before may end after this one's start
             float2 o[8];
             const float2* d = dst;
             int l = left;

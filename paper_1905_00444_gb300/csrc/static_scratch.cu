@@ -14,8 +14,8 @@
 // capture.
 //
 // All calls share the array and it keeps the last call's contents: each call copies the
-// plan's tables into it and clears the per-item header and the output before use, and
-// every other byte a call reads it has written first.  Calls that overlap on the GPU
+// plan's tables into it and writes every other byte that it reads first (a site's exponent
+// is stored or its maximum cleared, an output row begins with its first slice).  Calls that overlap on the GPU
 // (for example on two streams) race on the array.
 //
 // The tables are copied from the plan's own host image, which lives as long as the plan.
@@ -52,8 +52,6 @@ qfx_status scratch_address(void** out) {
   *out = g_addr[dev];
   return QFX_OK;
 }
-
-uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
 }  // namespace
 
