@@ -1258,6 +1258,11 @@ int ensure_tc_attr() {
       e = cudaFuncSetAttribute(cgemm_pair_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kMaxSmem - kStaticSmem);
     if (e != cudaSuccess) return (int)e;
+    // the roles' shares are drawn from what the launch gives: with fewer registers than that
+    // (another compiler's choice) the epilogue's warps would wait for theirs without end
+    cudaFuncAttributes fa{};
+    if ((e = cudaFuncGetAttributes(&fa, cgemm_pair_kernel<MODE>)) != cudaSuccess) return (int)e;
+    if (fa.numRegs < kRegLaunch) return (int)cudaErrorLaunchOutOfResources;
     attr_done[dev] = 1;
   }
   return 0;
