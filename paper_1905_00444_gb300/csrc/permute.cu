@@ -478,22 +478,18 @@ int launch_perm_tma(const PermTma& a, const CUtensorMap& map, float2* out, cudaS
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev0);
   cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev0);
   // Blocks per SM: more copies in flight crowd the stores, fewer leave the memory idle.  us with 4 /
-  // 6 / 8 blocks of two buffers, then with four buffers and as many blocks as fit (220 KB of shared
-  // memory are the limit):
-  //  - boxes of 8 KB take 4 where the output runs along la are long, and where la and lb are neighbours
-  //    in input and output, a batch of plain transposes: 16384 x 16384 651 / 836 / 847, 853; (64, 2^20)
-  //    173 / 187 / 195, 200;
-  //  - 6 where they are short (one tile of la, or two of 64): (27, 8, 64, 65, 16) to (0, 4, 1, 3, 2) 47 /
-  //    41 / 42, 44; (32, 64, 128, 64) to (2, 0, 3, 1) 54 / 47 / 50, 52;
-  //  - boxes of 16 KB take 4: seven axes reversed 340 / 400 / 400, 387;
-  //  - boxes below 8 KB (no axis with a factor 2 to box) need four buffers and all the blocks: (25,
-  //    32, 47, 2, 16, 32) to (3, 5, 1, 0, 2, 4) 155 / 127 / 111, 107; (4194304, 16) 324 / 247 / 214, 164;
-  //  - tiles cut off at the edge of la or lb copy less and take more blocks for the same bytes: (64, 2,
-  //    89, 69, 32) reversed, half of whose tiles are 5 of 64 wide, 113 / 99 / 92, 90; but not where la
-  //    has 16-wide tiles, whose short runs crowd the stores already: (64, 18, 64, 16, 32) to (0, 2, 3, 4,
-  //    1) 141 / 162 / 163, 153;
-  //  - what L2 holds, or nearly, is bound by latency and takes 8: (512, 106, 128) 22.6 / 19.9 / 18.5,
-  //    8192 x 1024 (134 MB in and out) 26.6 / 23.7 / 22.6; but 4096 x 4096 (268 MB) 46.9 / 51.9 / 53.4.
+  // 6 / 8 blocks of two buffers, then with four buffers and as many as 220 KB of shared memory hold:
+  //  - boxes of 8 KB or more take 4: 16384 x 16384 651 / 836 / 847, 853; seven axes reversed (16 KB) 340 /
+  //    400 / 400, 387; those of 8 KB 6 where the output runs along la are short (one tile of la, or two
+  //    of 64) and la and lb are not neighbours on both sides: (27, 8, 64, 65, 16) to (0, 4, 1, 3, 2)
+  //    47 / 41 / 42, 44;
+  //  - smaller boxes need four buffers and all the blocks: (25, 32, 47, 2, 16, 32) to (3, 5, 1, 0, 2, 4)
+  //    155 / 127 / 111, 107;
+  //  - tiles cut off at an edge copy less and take more blocks for the same bytes: (64, 2, 89, 69, 32)
+  //    reversed 113 / 99 / 92, 90; but not where la has 16-wide tiles, whose short runs crowd the
+  //    stores already: (64, 18, 64, 16, 32) to (0, 2, 3, 4, 1) 141 / 162 / 163, 153;
+  //  - what L2 holds, or nearly, is bound by latency and takes 8: 8192 x 1024 (134 MB in and out)
+  //    26.6 / 23.7 / 22.6; but 4096 x 4096 (268 MB) 46.9 / 51.9 / 53.4.
   const int64_t tile_el = (TA > 16 ? a.tiles_a * TA : a.Da) * a.tiles_b * 16, real_el = a.Da * a.Db;
   const bool in_l2 = 16 * real_el * a.nbatch * a.BZ * a.BY <= (int64_t)l2 * 3 / 2;
   const int box = 16 * TA * 8 * a.BZ * a.BY;
