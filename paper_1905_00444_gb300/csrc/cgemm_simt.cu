@@ -221,11 +221,11 @@ int num_sms() {
 // step takes the tile of least time.  A tile's times, alone on its SM and for each of those that
 // share one, are relative to 64 x 64 alone (105 us at K = 1024 and even Sd, 117 odd), for even and for
 // odd Sd; they are fitted to 1300 steps of K = 16 to 1024, N = 2 to 512, 64 to 80000 columns.  The
-// choice is 0.6% slower than each step's fastest tile on geometric mean, and 11% faster than the
+// choice is 0.2% slower than each step's fastest tile on geometric mean, and 11% faster than the
 // first tile that gives more CTAs than SMs (852 columns of K = 1024, N = 512: 106 us with 32 x 128 and
 // 112 CTAs, 136 with 16 x 128 and 224).  Where K < 32 loads and stores count more than the loop, and
 // CTAs that share an SM hide one another's: their times count 0.65 (all amplitudes of 4x4x(1+16+1)
-// 110.7 us, 113.4 without).
+// 110.7 us, 113.4 without; measured with slabs of 8 rows k in all tiles).
 // Every tile sums an output's k terms in the same order, so the choice never changes a result.
 int fill_variant(int variant, int64_t K, int64_t N, int64_t J, int batch) {
   struct Tile { int bm, bj, alone[2], shared[2]; };
@@ -233,8 +233,8 @@ int fill_variant(int variant, int64_t K, int64_t N, int64_t J, int batch) {
                                {32, 256, {217, 217}, {200, 200}}, {16, 256, {120, 140}, {125, 125}},
                                {8, 512, {145, 193}, {180, 180}}};
   static const Tile fill[5] = {{64, 64, {100, 100}, {97, 97}}, {32, 128, {102, 102}, {107, 107}},    // 20..24, 25..29
-                               {16, 128, {72, 72}, {74, 68}}, {8, 256, {85, 112}, {97, 80}},
-                               {8, 128, {53, 53}, {60, 54}}};
+                               {16, 128, {72, 72}, {74, 68}}, {8, 256, {73, 94}, {80, 80}},
+                               {8, 128, {44, 44}, {46, 46}}};
   if (variant < 0 || variant > 9 || batch < 1) return variant;
   const int64_t sms = num_sms();
   const int odd = variant >= 5;

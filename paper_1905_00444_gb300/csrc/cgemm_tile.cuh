@@ -9,7 +9,7 @@
 // FP32 CGEMM, without tensor cores).
 //
 // Tiling: one CTA computes BM x BJ outputs with NTH threads, each thread TM x TJ.  The k
-// loop moves BK = 8 slabs of S and B through two shared-memory buffers; the slab after the
+// loop moves slabs of S and B (8 rows k, or 16) through two shared-memory buffers; the slab after the
 // next waits in registers meanwhile.  B is stored with the real parts of two neighbouring
 // columns side by side and then their imaginary parts, so that a 16-byte read gives two
 // operands of the packed FP32 FMA (two columns per instruction); the entries of S become
@@ -22,7 +22,7 @@
 // with 8 slabs to a tile, gains most of its time from the second one.
 //
 // JMODE loads two columns as one 16-byte vector (Sd even).  KMODE takes any Sd: for Sd = 1
-// (the last site of a line) a column is contiguous in k and 8 lanes read its slab; otherwise
+// (the last site of a line) a column is contiguous in k and 8 lanes (or 16) read its slab; otherwise
 // the lanes run along s with 8-byte loads.
 #pragma once
 #include <cuda_runtime.h>
@@ -40,10 +40,12 @@ struct StepArgs {
   int32_t beta;   // 1: add the product into C (a chunk of a long contraction), 0: write it
 };
 
-constexpr int BK = 8;
-
 template <int BM, int BJ, int TM, int TJ, bool KMODE, int NTH = 256>
 struct Cfg {
+  // Rows k of a slab.  The fill tiles of 8 rows move 8 bytes for 64 FMAs and are bound by what they
+  // have in flight: a slab of 16 takes 1024 x 8 over 50000 columns from 151 to 122 us (Sd = 64) and 185
+  // to 144 (Sd = 1).  8 x 512 has no room for it beside a second CTA.
+  static constexpr int BK = BM == 8 && BJ <= 256 ? 16 : 8;
   static constexpr int TYN = BM / TM, TXN = BJ / TJ;
   static constexpr int LDA = BM + 2, LDB = BJ + 2;   // float2 per row; rows are 16-byte multiples
   static constexpr int A_IT = (BK * BM + NTH - 1) / NTH;
@@ -94,7 +96,7 @@ template <int BM, int BJ, int TM, int TJ, bool KMODE, int NTH = 256>
 __device__ __forceinline__ void cgemm_tile(const StepArgs& a, int64_t tile, int64_t item,
                                            float4* smem_raw) {
   using C_ = Cfg<BM, BJ, TM, TJ, KMODE, NTH>;
-  constexpr int TXN = C_::TXN, LDA = C_::LDA, LDB = C_::LDB, TQ = TJ / 2;
+  constexpr int BK = C_::BK, TXN = C_::TXN, LDA = C_::LDA, LDB = C_::LDB, TQ = TJ / 2;
   float2* As = reinterpret_cast<float2*>(smem_raw);
   float2* Bs = As + 2 * BK * LDA;
 
@@ -219,6 +221,8 @@ __device__ __forceinline__ void cgemm_tile(const StepArgs& a, int64_t tile, int6
     const float2* Bk = Bs + buf * BK * LDB + tx * 2;
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
+      // the padding of every tile ends at a multiple of 8
+      if (BK == 16 && kk == 8 && kt + 1 == KT && klast <= 8) break;
       float2 sv[TM];
       f32x2 br[TQ], bi[TQ];
 #pragma unroll

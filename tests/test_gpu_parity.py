@@ -350,6 +350,29 @@ def test_tile_of_a_small_grid(qfx, shape):
     qfx.sync()
 
 
+@pytest.mark.parametrize("sd", [1, 2, 7])
+@pytest.mark.parametrize("k", [1, 7, 8, 9, 15, 16, 17, 24, 25, 40, 47])
+def test_slabs_of_eight_row_tiles(qfx, k, sd):
+    """The small tiles of 8 rows take 16 rows k a slab, the others 8: last slabs of any length, on
+    the tile that the library chooses, the one that can be asked for and the usual one, bit for
+    bit, and against the definition within k + 2 roundings of the terms' sum."""
+    J, N = 1300, 7
+    P = J // sd
+    S = ri.random_complex(k * N, seed=21)
+    B = ri.random_complex(P * k * sd, seed=22)
+    d_S, d_B = torch.from_numpy(S).cuda(), torch.from_numpy(B).cuda()
+    odd = 5 * (sd % 2)
+    auto = qfx.contract_step(d_S, d_B, P, k, N, N, sd).cpu().numpy()
+    for v in (4 + odd, 23 + odd):
+        out = qfx.contract_step(d_S, d_B, P, k, N, N, sd, variant=v).cpu().numpy()
+        np.testing.assert_array_equal(auto, out)
+    qfx.sync()
+    S64, B64 = S.reshape(k, N).astype(np.complex128), B.reshape(P, k, sd).astype(np.complex128)
+    ref = np.einsum("kn,pks->pns", S64, B64)
+    scale = np.einsum("kn,pks->pns", abs(S64), abs(B64))
+    assert np.all(abs(auto.reshape(P, N, sd) - ref) <= 2 * (k + 2) * 2.0 ** -24 * 2 * scale)
+
+
 @pytest.mark.parametrize("case", [((16, 8, 3, 16), (3, 2, 1, 0)), ((16, 6, 5, 40), (3, 2, 1, 0)),
                                   ((16, 4, 24), (2, 1, 0)), ((32, 2, 7, 18), (3, 2, 1, 0)),
                                   ((2, 16, 3, 4, 32), (4, 2, 0, 3, 1)), ((4, 2, 32, 5, 16), (3, 4, 1, 0, 2)),
